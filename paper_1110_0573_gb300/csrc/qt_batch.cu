@@ -4,8 +4,9 @@
 // Persistent CTAs of 256 threads take work items from a device counter, in
 // the order the host sorted them (largest estimated cost first):
 //   * a master-equation item (paper section 3.1) is solved by the whole CTA
-//     with the team-generic solver of qt_me_impl.cuh (the team is the CTA;
-//     its Dormand-Prince buffers live in the CTA's slice of the workspace);
+//     with the solver of qt_me_small.cuh (its entry arrays in shared memory
+//     when they fit, else in the CTA's slice of the workspace), or, with wide
+//     operators, with the team-generic solver of qt_me_impl.cuh;
 //   * a Monte-Carlo item (paper section 3.2) is a block of trajectories of
 //     one problem; the CTA's eight warps take its trajectories one at a time
 //     and integrate them with the warp-group trajectory code of
@@ -14,6 +15,7 @@
 // CUDA graph.
 #include "qt_mc_impl.cuh"
 #include "qt_me_impl.cuh"
+#include "qt_me_small.cuh"
 
 namespace qt {
 
@@ -21,11 +23,25 @@ namespace {
 
 constexpr int kBatchWarps = kBatchBlock / 32;
 
-template <typename T>
-struct BatchShared {
+// Dynamic shared memory per CTA: two CTAs per SM for the mixed kernel, one
+// for the FP64 kernel.
+template <typename T> constexpr size_t kBatchSmem = sizeof(T) == 4 ? 112 * 1024 : 224 * 1024;
+
+// The CTA's current item, then one of: the Monte-Carlo items' buffers, the
+// general master-equation solver's scratch, the small solver's shared memory.
+struct BatchItemShared {
+  MeArgs me;
+  unsigned long long item;
+};
+constexpr size_t kBatchItemBytes = (sizeof(BatchItemShared) + 255) / 256 * 256;
+
+struct BatchMeShared {
   double sh[kMePartialMax * 8 + kMePartialMax];
   double tot[kMePartialMax];
-  MeArgs me;
+};
+
+template <typename T>
+struct BatchShared {
   McArgs mc[kBatchWarps];
   GroupScalars gs[kBatchWarps][2];  // one per trajectory group (half-warps when G = 16)
   typename CT<T>::V ybuf[kBatchWarps][128];  // per group two copies (Traj::publish)
@@ -33,8 +49,10 @@ struct BatchShared {
   typename CT<T>::V hlo[kBatchWarps][sizeof(T) == 4 ? 64 * 4 : 1];
   // mixed precision: each warp's two buffers of lo psi (64 rows each)
   typename CT<T>::V lpb[kBatchWarps][sizeof(T) == 4 ? 2 * 64 : 1];
-  unsigned long long item;
 };
+static_assert(kBatchItemBytes + sizeof(BatchShared<double>) <= kBatchSmem<double> &&
+                  kBatchItemBytes + sizeof(BatchShared<float>) <= kBatchSmem<float>,
+              "shared memory of the batched kernel");
 
 // Integrates the trajectories of one Monte-Carlo item on this warp: groups
 // of G lanes (the whole warp, or its two halves for small dimensions), each
@@ -86,16 +104,18 @@ __device__ void batch_mc_warp(const BatchArgs &a, const BatchProblem &P, const M
 
 template <typename T>
 __global__ void __launch_bounds__(kBatchBlock, (sizeof(T) == 4 ? 2 : 1)) batch_kernel(const __grid_constant__ BatchArgs a) {
-  __shared__ BatchShared<T> sm;
+  extern __shared__ __align__(256) unsigned char dyn[];
+  BatchItemShared &cur = *reinterpret_cast<BatchItemShared *>(dyn);
+  BatchShared<T> &sm = *reinterpret_cast<BatchShared<T> *>(dyn + kBatchItemBytes);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   for (;;) {
     if (threadIdx.x == 0) {
       unsigned long long it = atomicAdd(a.next_item, 1ULL);
       if (*(volatile int *)a.status != 0) it = (unsigned long long)a.n_items;
-      sm.item = it;
+      cur.item = it;
     }
     __syncthreads();
-    const unsigned long long it = sm.item;
+    const unsigned long long it = cur.item;
     __syncthreads();
     if (it >= (unsigned long long)a.n_items) break;
     const BatchItem item = a.items[it];
@@ -103,7 +123,7 @@ __global__ void __launch_bounds__(kBatchBlock, (sizeof(T) == 4 ? 2 : 1)) batch_k
     const int64_t out_off = P.expect_off * (int64_t)a.n_t;
     if (P.kind == QT_KIND_ME) {
       if (threadIdx.x == 0) {
-        MeArgs &m = sm.me;
+        MeArgs &m = cur.me;
         m.ops = P.ops;
         m.n_c = P.n_c;
         m.n_e = P.n_e;
@@ -125,13 +145,31 @@ __global__ void __launch_bounds__(kBatchBlock, (sizeof(T) == 4 ? 2 : 1)) batch_k
         m.rhs_in = nullptr;
         m.rhs_out = nullptr;
         m.n_td = 0;
+        m.small = P.small;
       }
       __syncthreads();
-      BlockTeam team;
-      SparseRhs<T> rhs(sm.me, sizeof(T) == 8
-                                  ? reinterpret_cast<const typename CT<T>::V *>(sm.me.ops.val64)
-                                  : reinterpret_cast<const typename CT<T>::V *>(sm.me.ops.val32));
-      me_solve<T>(sm.me, team, rhs, sm.sh, sm.tot);
+      const int prec = sizeof(T) == 4 ? QT_MIXED : QT_FP64;
+      const bool herm = P.state_is_ket != 0;
+      const int d = P.ops.d, nent = small_entries(d, herm);
+      unsigned char *region = dyn + kBatchItemBytes;
+      constexpr size_t room = kBatchSmem<T> - kBatchItemBytes;
+      const size_t base = small_smem(prec, d, nent, P.small, 1, kBatchBlock, false).total;
+      if (2 * P.small.nl + P.small.kc <= kSmallTerms && base <= room) {
+        // the entry arrays after the solver's shared memory when they fit
+        unsigned char *work =
+            base + small_ws_bytes(prec, d, nent, P.small, 1, kBatchBlock) <= room
+                ? region + base
+                : reinterpret_cast<unsigned char *>(cur.me.work);
+        SmallSolver<T, false, false> s(cur.me, herm, region, work, 0, 1);
+        s.solve();
+      } else {
+        BatchMeShared &g = *reinterpret_cast<BatchMeShared *>(region);
+        BlockTeam team;
+        SparseRhs<T> rhs(cur.me, sizeof(T) == 8
+                                     ? reinterpret_cast<const typename CT<T>::V *>(cur.me.ops.val64)
+                                     : reinterpret_cast<const typename CT<T>::V *>(cur.me.ops.val32));
+        me_solve<T>(cur.me, team, rhs, g.sh, g.tot);
+      }
       __syncthreads();
     } else {
       if (lane == 0) {
@@ -209,8 +247,11 @@ int grid_for_batch() {
   int dev = 0, sms = 0, per_sm = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return -1;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return -1;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_kernel<T>, kBatchBlock, 0) !=
-      cudaSuccess)
+  if (cudaFuncSetAttribute(batch_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)kBatchSmem<T>) != cudaSuccess)
+    return -1;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_kernel<T>, kBatchBlock,
+                                                    kBatchSmem<T>) != cudaSuccess)
     return -1;
   if (per_sm < 1) return -1;
   return sms * per_sm;
@@ -229,9 +270,9 @@ size_t batch_ws_stride(int dmax, int precision) {
 
 cudaError_t launch_batch(const BatchArgs &a, int precision, int grid, cudaStream_t s) {
   if (precision == QT_MIXED)
-    batch_kernel<float><<<grid, kBatchBlock, 0, s>>>(a);
+    batch_kernel<float><<<grid, kBatchBlock, kBatchSmem<float>, s>>>(a);
   else
-    batch_kernel<double><<<grid, kBatchBlock, 0, s>>>(a);
+    batch_kernel<double><<<grid, kBatchBlock, kBatchSmem<double>, s>>>(a);
   return cudaGetLastError();
 }
 

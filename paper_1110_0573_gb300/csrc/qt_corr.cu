@@ -4,8 +4,10 @@
 // solve, X_k = B rho(t_k) is evolved over tau by the same Lindblad generator
 // and C(t_k, tau_j) = Tr[A X_k(t_k + tau_j)].
 //
-// Small systems: one CTA per X_k (the general solver of qt_me_impl.cuh on a
-// CTA team), X_k and the shifted output times formed by the CTA itself.
+// Small systems: one CTA per X_k (the solver of qt_me_small.cuh on all d*d
+// entries; the general solver of qt_me_impl.cuh for the systems that it does
+// not take), X_k and the shifted output times formed by the CTA itself.  With
+// two CTAs per SM the dim-20 FP64 correlation keeps the FP64 pipe 80 % busy.
 // Larger systems: corr_prepare_kernel forms one X_k and its times, and the
 // cooperative solver of qt_me.cu evolves it.
 //
@@ -13,6 +15,7 @@
 // propagator): every matrix unit evolved, its states scattered into the
 // columns of U(t_k).
 #include "qt_me_impl.cuh"
+#include "qt_me_small.cuh"
 
 namespace qt {
 
@@ -48,19 +51,39 @@ __global__ void corr_prepare_kernel(const __grid_constant__ OpTable ops,
                (int64_t)gridDim.x * blockDim.x);
 }
 
+// How a CTA solves: the shared-memory solver of qt_me_small.cuh with the
+// entry arrays in shared memory or in the workspace, or the general solver
+// (time-dependent terms, wide operators).
+enum class SmallMode { kShared, kWork, kGeneral };
+
+template <typename T, SmallMode MODE>
+__device__ void cta_solve(const MeArgs &m) {
+  if constexpr (MODE == SmallMode::kGeneral) {
+    using V = typename CT<T>::V;
+    __shared__ double sh[kMePartialMax * (kMeBlock / 32) + kMePartialMax];
+    __shared__ double tot[kMePartialMax];
+    __shared__ double tdcoef[kTdMax];
+    BlockTeam team;
+    SparseRhs<T> rhs(m, sizeof(T) == 8 ? reinterpret_cast<const V *>(m.ops.val64)
+                                       : reinterpret_cast<const V *>(m.ops.val32), tdcoef);
+    me_solve<T>(m, team, rhs, sh, tot);
+  } else {
+    extern __shared__ double2 dyn_smem[];
+    SmallSolver<T, false, MODE == SmallMode::kShared> s(
+        m, false, reinterpret_cast<unsigned char *>(dyn_smem),
+        reinterpret_cast<unsigned char *>(m.work), 0, 1);
+    s.solve();
+  }
+}
+
 // CTA b evolves X_k for k = b, b + grid, ...; its slab of a.work holds the
 // solver workspace, X_k and the times.  a carries the tau evolution (n_t =
 // n_tau, expect = the correlation array, general solver).
-template <typename T>
+// MODE: the solver of the CTA (SmallMode below).
+template <typename T, SmallMode MODE>
 __global__ void __launch_bounds__(kMeBlock) corr_block_kernel(const __grid_constant__ MeArgs a,
                                                               const __grid_constant__ CorrArgs c) {
-  using V = typename CT<T>::V;
   __shared__ MeArgs m;
-  __shared__ double sh[kMePartialMax * (kMeBlock / 32) + kMePartialMax];
-  __shared__ double tot[kMePartialMax];
-  __shared__ double tdcoef[kTdMax];
-  const V *val = sizeof(T) == 8 ? reinterpret_cast<const V *>(a.ops.val64)
-                                : reinterpret_cast<const V *>(a.ops.val32);
   char *slab = reinterpret_cast<char *>(a.work) + (size_t)blockIdx.x * c.ws_stride;
   double2 *X = reinterpret_cast<double2 *>(slab + c.x_off);
   double *times = reinterpret_cast<double *>(slab + c.times_off);
@@ -74,9 +97,7 @@ __global__ void __launch_bounds__(kMeBlock) corr_block_kernel(const __grid_const
       m.work = slab;
     }
     __syncthreads();
-    BlockTeam team;
-    SparseRhs<T> rhs(m, val, tdcoef);
-    me_solve<T>(m, team, rhs, sh, tot);
+    cta_solve<T, MODE>(m);
     __syncthreads();  // m, X and times are rewritten for the next k
   }
 }
@@ -84,16 +105,10 @@ __global__ void __launch_bounds__(kMeBlock) corr_block_kernel(const __grid_const
 // The propagator: CTA b evolves the matrix units E_k (k = a d + b') for
 // k = b, b + grid, ... from tlist[0] by the general solver and scatters each
 // output state rho_k(t_m) into column k of U(t_m): U[m][ij][k].
-template <typename T>
+template <typename T, SmallMode MODE>
 __global__ void __launch_bounds__(kMeBlock) prop_block_kernel(const __grid_constant__ MeArgs a,
                                                               const __grid_constant__ PropArgs p) {
-  using V = typename CT<T>::V;
   __shared__ MeArgs m;
-  __shared__ double sh[kMePartialMax * (kMeBlock / 32) + kMePartialMax];
-  __shared__ double tot[kMePartialMax];
-  __shared__ double tdcoef[kTdMax];
-  const V *val = sizeof(T) == 8 ? reinterpret_cast<const V *>(a.ops.val64)
-                                : reinterpret_cast<const V *>(a.ops.val32);
   const int64_t n = (int64_t)a.ops.d * a.ops.d;
   char *slab = reinterpret_cast<char *>(a.work) + (size_t)blockIdx.x * p.ws_stride;
   double2 *X = reinterpret_cast<double2 *>(slab + p.x_off);
@@ -108,9 +123,7 @@ __global__ void __launch_bounds__(kMeBlock) prop_block_kernel(const __grid_const
       m.work = slab;
     }
     __syncthreads();
-    BlockTeam team;
-    SparseRhs<T> rhs(m, val, tdcoef);
-    me_solve<T>(m, team, rhs, sh, tot);
+    cta_solve<T, MODE>(m);
     __syncthreads();
     for (int t = 0; t < a.n_t; ++t)
       for (int64_t idx = threadIdx.x; idx < n; idx += blockDim.x)
@@ -119,58 +132,95 @@ __global__ void __launch_bounds__(kMeBlock) prop_block_kernel(const __grid_const
   }
 }
 
-template <typename T>
-int prop_grid_t(int64_t units) {
+// The mode and the dynamic shared memory of a system (general matrices: all
+// d*d entries).
+SmallMode small_mode(const MeArgs &a, int precision, size_t *smem) {
+  *smem = 0;
+  if (!small_fits(a)) return SmallMode::kGeneral;
+  const int d = a.ops.d, nent = small_entries(d, false);
+  *smem = small_smem(precision, d, nent, a.small, 1, kMeBlock, true).total;
+  if (*smem <= kSmallSmemMax) return SmallMode::kShared;
+  *smem = small_smem(precision, d, nent, a.small, 1, kMeBlock, false).total;
+  return SmallMode::kWork;
+}
+
+// Resident CTAs of a kernel with smem bytes of dynamic shared memory, at most
+// units (negative on error).
+template <typename K>
+int block_grid(K kern, size_t smem, int64_t units) {
   int dev = 0, sms = 0, per_sm = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return -1;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return -1;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, prop_block_kernel<T>, kMeBlock, 0) !=
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
       cudaSuccess)
+    return -1;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kMeBlock, smem) != cudaSuccess)
     return -1;
   if (per_sm < 1) return -1;
   const int64_t cap = (int64_t)sms * per_sm;
   return (int)(units < cap ? units : cap);
 }
 
-template <typename T>
-int corr_grid_t(int n_t) {
-  int dev = 0, sms = 0, per_sm = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return -1;
-  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return -1;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, corr_block_kernel<T>, kMeBlock, 0) !=
-      cudaSuccess)
-    return -1;
-  if (per_sm < 1) return -1;
-  const int cap = sms * per_sm;
-  return n_t < cap ? n_t : cap;
+// fn(kernel) for the instance of the given precision and mode.
+template <typename F>
+auto with_corr_kernel(int precision, SmallMode m, F &&fn) {
+  if (precision == QT_MIXED)
+    return m == SmallMode::kShared  ? fn(corr_block_kernel<float, SmallMode::kShared>)
+           : m == SmallMode::kWork  ? fn(corr_block_kernel<float, SmallMode::kWork>)
+                                    : fn(corr_block_kernel<float, SmallMode::kGeneral>);
+  return m == SmallMode::kShared ? fn(corr_block_kernel<double, SmallMode::kShared>)
+         : m == SmallMode::kWork ? fn(corr_block_kernel<double, SmallMode::kWork>)
+                                 : fn(corr_block_kernel<double, SmallMode::kGeneral>);
+}
+template <typename F>
+auto with_prop_kernel(int precision, SmallMode m, F &&fn) {
+  if (precision == QT_MIXED)
+    return m == SmallMode::kShared  ? fn(prop_block_kernel<float, SmallMode::kShared>)
+           : m == SmallMode::kWork  ? fn(prop_block_kernel<float, SmallMode::kWork>)
+                                    : fn(prop_block_kernel<float, SmallMode::kGeneral>);
+  return m == SmallMode::kShared ? fn(prop_block_kernel<double, SmallMode::kShared>)
+         : m == SmallMode::kWork ? fn(prop_block_kernel<double, SmallMode::kWork>)
+                                 : fn(prop_block_kernel<double, SmallMode::kGeneral>);
 }
 
 }  // namespace
 
-int corr_block_grid(int n_t, int precision) {
-  return precision == QT_MIXED ? corr_grid_t<float>(n_t) : corr_grid_t<double>(n_t);
+int corr_block_grid(const MeArgs &a, int n_t, int precision) {
+  size_t smem;
+  const SmallMode m = small_mode(a, precision, &smem);
+  return with_corr_kernel(precision, m, [&](auto *k) { return block_grid(k, smem, n_t); });
 }
 
 cudaError_t launch_corr_block(const MeArgs &a, const CorrArgs &c, int grid, int precision,
                               cudaStream_t s) {
-  if (precision == QT_MIXED)
-    corr_block_kernel<float><<<grid, kMeBlock, 0, s>>>(a, c);
-  else
-    corr_block_kernel<double><<<grid, kMeBlock, 0, s>>>(a, c);
-  return cudaGetLastError();
+  size_t smem;
+  const SmallMode m = small_mode(a, precision, &smem);
+  return with_corr_kernel(precision, m, [&](auto *k) {
+    cudaError_t e =
+        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    k<<<grid, kMeBlock, smem, s>>>(a, c);
+    return cudaGetLastError();
+  });
 }
 
-int prop_block_grid(int64_t units, int precision) {
-  return precision == QT_MIXED ? prop_grid_t<float>(units) : prop_grid_t<double>(units);
+int prop_block_grid(const MeArgs &a, int64_t units, int precision) {
+  size_t smem;
+  const SmallMode m = small_mode(a, precision, &smem);
+  return with_prop_kernel(precision, m, [&](auto *k) { return block_grid(k, smem, units); });
 }
 
 cudaError_t launch_prop_block(const MeArgs &a, const PropArgs &p, int grid, int precision,
                               cudaStream_t s) {
-  if (precision == QT_MIXED)
-    prop_block_kernel<float><<<grid, kMeBlock, 0, s>>>(a, p);
-  else
-    prop_block_kernel<double><<<grid, kMeBlock, 0, s>>>(a, p);
-  return cudaGetLastError();
+  size_t smem;
+  const SmallMode m = small_mode(a, precision, &smem);
+  return with_prop_kernel(precision, m, [&](auto *k) {
+    cudaError_t e =
+        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    k<<<grid, kMeBlock, smem, s>>>(a, p);
+    return cudaGetLastError();
+  });
 }
 
 cudaError_t launch_corr_prepare(const OpTable &ops, const CorrArgs &c, int k, double2 *X,

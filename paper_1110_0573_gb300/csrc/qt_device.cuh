@@ -195,6 +195,39 @@ template <> struct DPW<float> {
                          e7 = (float)(-(dp_r32(DP::e1) + dp_r32(DP::e3) + dp_r32(DP::e4) + dp_r32(DP::e5) + dp_r32(DP::e6)));
 };
 
+// The same pair for a linear right-hand side f(y) = L y that does not depend
+// on time, in powers of L: with v_k = L v_(k-1), v_0 = y, every stage is a
+// polynomial in h L, and the tableau above multiplied out gives
+//   ynew = y + sum_k c_k h^k v_k,                    k = 1..6,
+//   error = sum_k e_k h^k v_k + e_7 h L ynew
+// (the low orders of the error cancel against L ynew).  Six products per step
+// as before, but no stage combinations: 13 multiply-adds per component and
+// step instead of 33.
+struct DPP {
+  static constexpr double c2 = 1.0 / 2, c3 = 1.0 / 6, c4 = 1.0 / 24, c5 = 1.0 / 120,
+                          c6 = 1.0 / 600;  // c_1 = 1
+  static constexpr double e1 = 1.0 / 40, e2 = 1.0 / 40, e3 = 1.0 / 80, e4 = 1.0 / 240,
+                          e5 = 7.0 / 30000, e6 = 1.0 / 1875, e7 = -1.0 / 40;
+};
+__host__ __device__ constexpr double dpp_c(int k) {
+  return k == 1 ? 1.0 : k == 2 ? DPP::c2 : k == 3 ? DPP::c3 : k == 4 ? DPP::c4 : k == 5 ? DPP::c5 : DPP::c6;
+}
+__host__ __device__ constexpr double dpp_e(int k) {
+  return k == 1 ? DPP::e1 : k == 2 ? DPP::e2 : k == 3 ? DPP::e3 : k == 4 ? DPP::e4
+       : k == 5 ? DPP::e5 : k == 6 ? DPP::e6 : DPP::e7;
+}
+
+// a < b for values that are not negative, by their integer order (an FP64
+// comparison would go to the FP64 pipe).
+__device__ __forceinline__ bool pos_less(double a, double b) {
+  return __double_as_longlong(a) < __double_as_longlong(b);
+}
+
+__device__ __forceinline__ bool finite_bits(double x) {
+  return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000;
+}
+__device__ __forceinline__ bool finite_bits(float x) { return isfinite(x); }
+
 // Step-size controller shared by both solvers (see qt.h): returns the next
 // proposal after a step of length h with error norm err.
 __device__ __forceinline__ double dp_control(double h, double err, bool accepted,
@@ -207,6 +240,62 @@ __device__ __forceinline__ double dp_control(double h, double err, bool accepted
     return hn;
   }
   return h * fmax(0.2, 0.9 * pow(err, -0.2));
+}
+
+// 1 / x.  FP64: one third-order Householder step from the hardware's
+// approximate reciprocal (about 20 bits), three multiply-adds, within an ulp
+// or two; numbers whose reciprocal or approximation leaves the normal range
+// are divided.  An FP64 division costs about three times as many FP64
+// instructions, and those bound the FP64 solvers.
+__device__ __forceinline__ float recip(float x) { return rcp_approx(x); }
+__device__ __forceinline__ double recip(double x) {
+  const int hi = __double2hiint(x) & 0x7fffffff;
+  if (hi < 0x01000000 || hi >= 0x7e000000) return 1.0 / x;  // 2^-1007 .. 2^993
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-x, y, 1.0);
+  return fma(y, fma(e, e, e), y);
+}
+
+// x^(-1/10) for x in [1e-30, 1e30] from an FP32 value with relative error e:
+// one third-order Newton-Schroeder step, with r = 1 - x y^10,
+// y (1 + r / 10 + 11 r^2 / 200), which leaves about 40 e^3 (e = 1e-6), in
+// nine FP64 operations instead of a pow of the square root.
+__device__ __forceinline__ double inv_root10(double x, float seed) {
+  const double y = (double)seed;
+  const double y2 = y * y, y4 = y2 * y2, y8 = y4 * y4;
+  const double r = fma(-x, y8 * y2, 1.0);
+  return fma(y * r, fma(r, 0.055, 0.1), y);
+}
+
+// max(|a|, |b|), by the integer order of the magnitudes (an FP64 comparison
+// would go to the FP64 pipe).
+__device__ __forceinline__ double max_abs(double a, double b) {
+  const long long x = __double_as_longlong(a) & 0x7fffffffffffffffll;
+  const long long y = __double_as_longlong(b) & 0x7fffffffffffffffll;
+  return __longlong_as_double(x > y ? x : y);
+}
+__device__ __forceinline__ float max_abs(float a, float b) { return fmaxf(fabsf(a), fabsf(b)); }
+
+// dp_control with the squared error norm x = err^2 (err^(-1/5) = x^(-1/10)).
+// The FP32 form evaluates the factor in FP32, as the mixed solvers do.
+template <typename T>
+__device__ __forceinline__ double dp_control_sq(double h, double x, bool accepted,
+                                                bool after_reject, bool clipped, double hprop) {
+  const double facmax = !accepted || after_reject ? 1.0 : 5.0;
+  const float pf = ex2_approx(-0.1f * lg2_approx((float)x));
+  double fac;
+  if (!(pf < 6.f)) {  // err^2 below 1.6e-8 (or zero): far above the largest factor
+    fac = facmax;
+  } else if (!(pf > 0.2f)) {
+    fac = 0.2;
+  } else {
+    fac = 0.9 * (sizeof(T) == 8 ? inv_root10(x, pf) : (double)pf);
+    if (pos_less(fac, 0.2)) fac = 0.2;
+    if (pos_less(facmax, fac)) fac = facmax;
+  }
+  const double hn = h * fac;
+  return accepted && clipped && pos_less(hn, hprop) ? hprop : hn;
 }
 
 __device__ __forceinline__ double dp_hmin(double t, double tnext) {

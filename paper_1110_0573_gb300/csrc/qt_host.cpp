@@ -374,6 +374,36 @@ int ell_append(const Csr &A, std::vector<int> &cols, std::vector<double2> &vals,
   return w;
 }
 
+// Structure of H_eff and the collapse operators for the small-system solver;
+// a collapse operator's ELL width is its longest row, at least 1.
+qt::SmallInfo small_info(const Csr &heff, const std::vector<Csr> &C) {
+  qt::SmallInfo f = {0, 0, 1, 1};
+  for (int i = 0; i < heff.d; ++i) {
+    int n = 0;
+    for (int64_t p = heff.ptr[i]; p < heff.ptr[i + 1]; ++p)
+      if (heff.col[p] != i) {
+        ++n;
+        if (heff.val[p].imag() != 0.0) f.hreal = 0;
+      }
+    f.nl = std::max(f.nl, n);
+  }
+  for (const Csr &c : C) {
+    int w = 1;
+    bool diag = true, real = true;
+    for (int i = 0; i < c.d; ++i) {
+      w = std::max(w, (int)(c.ptr[i + 1] - c.ptr[i]));
+      for (int64_t p = c.ptr[i]; p < c.ptr[i + 1]; ++p) {
+        diag = diag && c.col[p] == i;
+        real = real && c.val[p].imag() == 0.0;
+      }
+    }
+    if (diag) continue;
+    f.kc += w * w;
+    if (!real) f.creal = 0;
+  }
+  return f;
+}
+
 int check_opts(const qt_opts *o) {
   if (!o) return fail(QT_EINVAL, "null options");
   if (!(o->rtol > 0.0) || !(o->atol >= 0.0) || !std::isfinite(o->rtol) || !std::isfinite(o->atol))
@@ -455,6 +485,7 @@ struct qt_system_s {
   void *ivl = nullptr;
   int ivl_cap = 0;
   int dict_gend[qt::kDictMaxGroups] = {};
+  qt::SmallInfo small = {};
 
   qt::OpTable table() const {
     qt::OpTable t;
@@ -568,6 +599,7 @@ void me_args(qt_system s, const qt_opts *o, int grid, void *ws, qt::MeArgs &a) {
   a.td_v = s->td_v_dev;
   a.n_cslots = s->n_cslots;
   a.n_cterms = s->n_cterms;
+  a.small = s->small;
   const size_t elem = o->precision == QT_MIXED ? sizeof(float2) : sizeof(double2);
   const size_t state_bytes = 11 * (size_t)s->d * s->d * elem;
   a.partial = reinterpret_cast<double *>(reinterpret_cast<char *>(ws) +
@@ -585,7 +617,9 @@ int ensure_dense(qt_system s);
 //                   or for a matrix the kernel finds Hermitian (else general);
 //   QT_ME_DENSE_TC  the Hermitian solver with the tensor-core product
 //                   (QT_ENONHERM from the device for a non-Hermitian matrix).
-// Sparse solves of dimension <= kMeSmallDim run the general solver on one CTA.
+// Sparse solves of dimension <= kMeSmallDim run on one CTA or cluster (the
+// solver of qt_me_small.cuh; QT_ME_AUTO evaluates the upper triangle only when
+// the initial state is a ket).
 int me_setup(qt_system s, const qt_opts *o, bool is_ket, qt::MeArgs &a) {
   const bool dense = o->me_method == QT_ME_DENSE_TC;
   const bool small = !dense && s->d <= qt::kMeSmallDim;
@@ -601,10 +635,17 @@ int me_setup(qt_system s, const qt_opts *o, bool is_ket, qt::MeArgs &a) {
                  : (herm ? qt::me_herm_grid(s->d, o->precision, s->n_cslots, s->n_cterms)
                          : qt::me_grid(s->d, o->precision));
   if (grid <= 0) return fail(QT_ECUDA, "cannot size the cooperative launch");
-  if ((rc = ensure_ws(s, qt::me_workspace_bytes(s->d, o->precision, grid)))) return rc;
+  const bool small_herm = small && is_ket && o->me_method == QT_ME_AUTO;
+  size_t ws = qt::me_workspace_bytes(s->d, o->precision, grid);
+  if (small) {
+    me_args(s, o, grid, nullptr, a);
+    ws = std::max(ws, qt::small_workspace_bytes(a, o->precision, small_herm, true));
+  }
+  if ((rc = ensure_ws(s, ws))) return rc;
   me_args(s, o, grid, s->ws, a);
   a.herm = herm ? (is_ket ? 1 : 2) : 0;
   a.single_cta = small ? 1 : 0;
+  a.small_herm = small_herm ? 1 : 0;
   return QT_OK;
 }
 
@@ -875,6 +916,7 @@ int qt_system_create_td(const qt_op *H, const qt_td *td, const qt_op *c_ops, int
     s->w_host.push_back(ell_append(A, cols, vals, diag_slot));
   };
   const Csr heff = effective_hamiltonian(Hc, C);
+  if (d <= qt::kMeSmallDim) s->small = small_info(heff, C);
   add(heff, true);
   DictOp dict;
   const bool have_dict = d > 128 && d <= 2048 && dictionary_form(heff, qt::kDictMaxValues, dict);
@@ -1149,12 +1191,16 @@ int qt_correlation_2op_2t_dev(qt_system s, const qt_c128 *state0_dev, int state_
   // store: rho(t_k) [n_t][d][d], the first solve's expectation values, then
   // either one CTA slab per CTA of the batched launch or one X_k + times
   const bool small = d <= qt::kMeSmallDim;
-  const int grid = small ? qt::corr_block_grid(n_t, o->precision) : 0;
+  qt::MeArgs a, b;
+  qt_opts o2 = *o;
+  if (o2.me_method == QT_ME_DENSE_TC) o2.me_method = QT_ME_AUTO;
+  me_args(s, &o2, 1, nullptr, b);
+  const int grid = small ? qt::corr_block_grid(b, n_t, o->precision) : 0;
   if (small && grid <= 0) return fail(QT_ECUDA, "cannot size the correlation launch");
   const size_t elem = o->precision == QT_MIXED ? sizeof(float2) : sizeof(double2);
   qt::CorrArgs c;
   std::memset(&c, 0, sizeof c);
-  c.x_off = up(11 * n * elem);
+  c.x_off = up(std::max(11 * n * elem, small ? qt::small_workspace_bytes(b, o->precision, false, false) : 0));
   c.times_off = c.x_off + up(n * sizeof(double2));
   c.ws_stride = c.times_off + up((size_t)n_tau * sizeof(double));
   const size_t states_bytes = up((size_t)n_t * n * sizeof(double2));
@@ -1175,9 +1221,6 @@ int qt_correlation_2op_2t_dev(qt_system s, const qt_c128 *state0_dev, int state_
   // X_k = B rho(t_k) over tau: the general solver (X_k is not Hermitian).
   // Both solves' workspace is sized before the first launch (a later growth
   // would free memory that the first solve may still be using).
-  qt_opts o2 = *o;
-  if (o2.me_method == QT_ME_DENSE_TC) o2.me_method = QT_ME_AUTO;
-  qt::MeArgs a, b;
   if (!small && (rc = me_setup(s, &o2, false, b))) return rc;
   void *ws_before = s->ws;
   if ((rc = me_setup(s, o, state_is_ket != 0, a))) return rc;
@@ -1384,19 +1427,20 @@ int qt_propagator_dev(qt_system s, const double *tlist_dev, int n_t, const qt_op
                 qt::kMeSmallDim);
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   const int64_t n = (int64_t)d * d;
-  const int grid = qt::prop_block_grid(n, o->precision);
+  qt_opts o2 = *o;
+  if (o2.me_method == QT_ME_DENSE_TC) o2.me_method = QT_ME_AUTO;
+  qt::MeArgs a;
+  me_args(s, &o2, 1, nullptr, a);
+  const int grid = qt::prop_block_grid(a, n, o->precision);
   if (grid <= 0) return fail(QT_ECUDA, "cannot size the propagator launch");
   auto up = [](size_t b) { return (b + 255) / 256 * 256; };
   const size_t elem = o->precision == QT_MIXED ? sizeof(float2) : sizeof(double2);
   qt::PropArgs p;
   p.U = reinterpret_cast<double2 *>(U_dev);
-  p.x_off = up(11 * (size_t)n * elem);
+  p.x_off = up(std::max(11 * (size_t)n * elem, qt::small_workspace_bytes(a, o->precision, false, false)));
   p.st_off = p.x_off + up((size_t)n * sizeof(double2));
   p.ws_stride = p.st_off + up((size_t)n_t * n * sizeof(double2));
   if ((rc = ensure_aux(s, (size_t)grid * p.ws_stride))) return rc;
-  qt_opts o2 = *o;
-  if (o2.me_method == QT_ME_DENSE_TC) o2.me_method = QT_ME_AUTO;
-  qt::MeArgs a;
   me_args(s, &o2, 1, s->aux, a);
   a.n_t = n_t;
   a.tlist = tlist_dev;
@@ -1578,6 +1622,7 @@ int qt_batch_create(const qt_problem *problems, int n_problems, qt_batch *out) {
     int64_t sbase;
   };
   std::vector<PInfo> info(n_problems);
+  std::vector<qt::SmallInfo> infos;
   qt_batch b = new (std::nothrow) qt_batch_s();
   if (!b) return fail(QT_ENOMEM, "host allocation");
   b->n = n_problems;
@@ -1658,6 +1703,7 @@ int qt_batch_create(const qt_problem *problems, int n_problems, qt_batch *out) {
     b->expect_base.push_back(b->expect_units);
     b->expect_units += P.n_e;
     b->me_cost.push_back((double)d * d * (2.0 * w_all[pi.wbase] + wsum_c2));
+    infos.push_back(small_info(He, C));
     b->mc_cost_per_traj.push_back(2.0 * d * w_all[pi.wbase]);
     b->dmax = std::max(b->dmax, d);
     item_bound += (P.kind == QT_KIND_ME) ? 1 : (nt + 31) / 32;
@@ -1708,6 +1754,7 @@ int qt_batch_create(const qt_problem *problems, int n_problems, qt_batch *out) {
     q.seed = problems[p].seed;
     q.state0 = st_dev + pi.sbase;
     q.expect_off = b->expect_base[p];
+    q.small = infos[p];
   }
   b->probs = (qt::BatchProblem *)up(probs.data(), probs.size() * sizeof(qt::BatchProblem));
   b->items_cap = (int)std::max<int64_t>(item_bound, 1);
@@ -1719,6 +1766,15 @@ int qt_batch_create(const qt_problem *problems, int n_problems, qt_batch *out) {
   const int g64 = qt::batch_grid(QT_FP64), g32 = qt::batch_grid(QT_MIXED);
   b->grid = std::max(g64, g32);
   b->ws_stride = qt::batch_ws_stride(b->dmax, QT_FP64);
+  for (int p = 0; p < n_problems; ++p) {  // and the small solver's workspace
+    if (problems[p].kind != QT_KIND_ME) continue;
+    qt::MeArgs m;
+    std::memset(&m, 0, sizeof m);
+    m.ops.d = info[p].d;
+    m.small = infos[p];
+    b->ws_stride = std::max(b->ws_stride, (qt::small_workspace_bytes(m, QT_FP64, probs[p].state_is_ket != 0,
+                                                                     false) + 255) / 256 * 256);
+  }
   if (b->grid <= 0) {
     delete b;
     return fail(QT_ECUDA, "cannot size the batch launch");

@@ -91,6 +91,16 @@ struct McArgs {
 constexpr int kDictMaxValues = 1024;
 constexpr int kDictMaxGroups = 16;
 
+// Structure of a system's operators, as the small-system solver
+// (qt_me_small.cuh) lays them out.  A collapse operator is diagonal when all
+// its entries are.
+struct SmallInfo {
+  int nl;     // most off-diagonal entries in a row of H_eff
+  int kc;     // sum of squared ELL widths of the collapse operators that are not diagonal
+  int hreal;  // every off-diagonal entry of H_eff is real
+  int creal;  // every entry of those collapse operators is real
+};
+
 // Kernel arguments of the master-equation solver.
 struct MeArgs {
   OpTable ops;
@@ -121,7 +131,9 @@ struct MeArgs {
   int n_td, td_op0;              // time-dependent terms (0: none), as in McArgs
   const int64_t *td_off;
   const double *td_t, *td_v;
-  int single_cta;                // 1: one CTA solves (small systems; no grid barriers)
+  int single_cta;                // 1: one CTA or cluster solves (small systems; no grid barriers)
+  SmallInfo small;               // structure of the operators for the small solver
+  int small_herm;                // small systems: evaluate the upper triangle (Hermitian state)
   int herm;                      // 0: general solver (no symmetry assumed);
                                  // 1: Hermitian solver (state0 is a ket or Hermitian);
                                  // 2: test the initial matrix on the device, then choose
@@ -223,6 +235,7 @@ struct BatchProblem {
   uint64_t seed;
   const double2 *state0;  // ME: ket or rho0; MC: normalised ket
   int64_t expect_off;     // offset of the outputs (per unit n_t: off = base * n_t)
+  SmallInfo small;
 };
 
 // A work item: a master-equation problem, or a block of trajectories.
@@ -318,10 +331,10 @@ cudaError_t launch_identity_state(double2 *rho, int d, cudaStream_t s);
 cudaError_t launch_set_status(int *status, int code, cudaStream_t s);  // first error wins
 cudaError_t launch_diff_norm(const double2 *a, const double2 *b, int64_t n, double *out,
                              cudaStream_t s);
-int prop_block_grid(int64_t units, int precision);  // CTAs of the propagator launch
+int prop_block_grid(const MeArgs &a, int64_t units, int precision);  // CTAs of the propagator launch
 cudaError_t launch_prop_block(const MeArgs &a, const PropArgs &p, int grid, int precision,
                               cudaStream_t s);
-int corr_block_grid(int n_t, int precision);  // CTAs of the batched small-system launch
+int corr_block_grid(const MeArgs &a, int n_t, int precision);  // CTAs of the batched small-system launch
 cudaError_t launch_corr_block(const MeArgs &a, const CorrArgs &c, int grid, int precision,
                               cudaStream_t s);
 cudaError_t launch_corr_prepare(const OpTable &ops, const CorrArgs &c, int k, double2 *X,
@@ -337,6 +350,9 @@ cudaError_t launch_normalise(const double2 *in, double2 *out, int d, int *status
                              cudaStream_t s, const double *tlist = nullptr, int n_t = 0,
                              double *ivl_tb = nullptr, float *ivl_len = nullptr);
 size_t me_workspace_bytes(int d, int precision, int grid);
+// Workspace of the small-system solver on one CTA or (cluster) as launch_me
+// runs it; 0 for systems it does not take.
+size_t small_workspace_bytes(const MeArgs &a, int precision, bool herm, bool cluster);
 
 // Records msg as the calling thread's last error and returns code.
 int set_error(int code, const char *msg);

@@ -3,6 +3,7 @@
 // product on the CUDA cores, or the general solver of qt_me_impl.cuh (no
 // symmetry assumed) for non-Hermitian initial matrices and on request.
 #include "qt_me_herm.cuh"
+#include "qt_me_small.cuh"
 
 namespace qt {
 
@@ -39,8 +40,29 @@ __global__ void __launch_bounds__(kMeBlock) me_kernel(const __grid_constant__ Me
   }
 }
 
-// Small systems: the general solver on one CTA (team barriers are
-// __syncthreads, no grid-wide synchronisation).
+// Small systems: the whole solve on one CTA (CL = false) or one cluster.
+template <typename T, bool CL, bool KS>
+__global__ void __launch_bounds__(kMeBlock, 1) me_small_kernel(const __grid_constant__ MeArgs a) {
+  extern __shared__ double2 dyn_smem[];
+  int rank = 0, nranks = 1;
+  if constexpr (CL) {
+    rank = (int)cg::this_cluster().block_rank();
+    nranks = (int)cg::this_cluster().num_blocks();
+  }
+  unsigned char *work = nullptr;
+  if constexpr (!KS)
+    work = reinterpret_cast<unsigned char *>(a.work) +
+           rank * small_ws_bytes(sizeof(T) == 4 ? QT_MIXED : QT_FP64, a.ops.d,
+                                 small_entries(a.ops.d, a.small_herm != 0), a.small, nranks,
+                                 (int)blockDim.x);
+  SmallSolver<T, CL, KS> s(a, a.small_herm != 0, reinterpret_cast<unsigned char *>(dyn_smem), work,
+                           rank, nranks);
+  s.solve();
+}
+
+// Small systems with time-dependent terms, with operators too wide for the
+// shared-memory copy, and single right-hand sides: the general solver on one
+// CTA (team barriers are __syncthreads, no grid-wide synchronisation).
 template <typename T>
 __global__ void __launch_bounds__(kMeBlock) me_block_kernel(const __grid_constant__ MeArgs a) {
   using V = typename CT<T>::V;
@@ -98,9 +120,57 @@ size_t me_workspace_bytes(int d, int precision, int grid) {
   return 11 * (size_t)d * d * elem + (size_t)grid * kMePartialMax * sizeof(double) + 256;
 }
 
+// Workspace of the small solver for a system it takes (0: it does not).
+size_t small_workspace_bytes(const MeArgs &a, int precision, bool herm, bool cluster) {
+  if (!small_fits(a)) return 0;
+  const int d = a.ops.d, nent = small_entries(d, herm), ranks = cluster ? small_ranks(nent) : 1;
+  return ranks * small_ws_bytes(precision, d, nent, a.small, ranks, kMeBlock);
+}
+
+namespace {
+
+template <typename T, bool CL, bool KS>
+cudaError_t launch_small_inst(const MeArgs &a, size_t smem, int ranks, cudaStream_t s) {
+  cudaError_t e = cudaFuncSetAttribute(me_small_kernel<T, CL, KS>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(ranks);
+  cfg.blockDim = dim3(kMeBlock);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = ranks;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = CL ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, me_small_kernel<T, CL, KS>, a);
+}
+
+template <typename T>
+cudaError_t launch_small(const MeArgs &a, cudaStream_t s) {
+  const int prec = sizeof(T) == 4 ? QT_MIXED : QT_FP64;
+  const int d = a.ops.d, nent = small_entries(d, a.small_herm != 0);
+  const int ranks = small_ranks(nent);
+  for (int ks = 1; ks >= 0; --ks) {
+    const size_t smem = small_smem(prec, d, nent, a.small, ranks, kMeBlock, ks != 0).total;
+    if (smem > kSmallSmemMax) continue;
+    if (ranks > 1)
+      return ks ? launch_small_inst<T, true, true>(a, smem, ranks, s)
+                : launch_small_inst<T, true, false>(a, smem, ranks, s);
+    return ks ? launch_small_inst<T, false, true>(a, smem, ranks, s)
+              : launch_small_inst<T, false, false>(a, smem, ranks, s);
+  }
+  return cudaErrorInvalidValue;  // the matrices of kMeSmallDim always fit
+}
+
+}  // namespace
+
 template <typename T>
 cudaError_t launch_me_t(const MeArgs &a, cudaStream_t s) {
   if (a.single_cta) {
+    if (!a.rhs_in && small_fits(a)) return launch_small<T>(a, s);
     me_block_kernel<T><<<1, kMeBlock, 0, s>>>(a);
     return cudaGetLastError();
   }
