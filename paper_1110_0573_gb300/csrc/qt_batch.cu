@@ -176,6 +176,7 @@ __global__ void __launch_bounds__(kBatchBlock, (sizeof(T) == 4 ? 2 : 1)) batch_k
         McArgs &m = sm.mc[warp];
         m.ops = P.ops;
         m.heff_w = 0;
+        m.hreal = P.small.hreal;
         m.stage_aux = 0;
         m.aux_begin = 0;
         m.aux_slots = 0;

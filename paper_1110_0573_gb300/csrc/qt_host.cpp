@@ -916,7 +916,7 @@ int qt_system_create_td(const qt_op *H, const qt_td *td, const qt_op *c_ops, int
     s->w_host.push_back(ell_append(A, cols, vals, diag_slot));
   };
   const Csr heff = effective_hamiltonian(Hc, C);
-  if (d <= qt::kMeSmallDim) s->small = small_info(heff, C);
+  if (d <= 128) s->small = small_info(heff, C);  // the register Monte-Carlo instances use it too
   add(heff, true);
   DictOp dict;
   const bool have_dict = d > 128 && d <= 2048 && dictionary_form(heff, qt::kDictMaxValues, dict);
@@ -1078,6 +1078,7 @@ int qt_mcsolve_dev(qt_system s, const qt_c128 *psi0_dev, const double *tlist_dev
   a.ivl_len = ivl_len;
   a.ops = s->table();
   a.heff_w = s->w_host[0];
+  a.hreal = s->small.hreal;
   a.aux_begin = s->n_ops > 1 ? s->off_host[1] : s->total_slots;
   a.aux_slots = s->total_slots - a.aux_begin;
   a.n_c = s->n_c;

@@ -38,6 +38,7 @@ constexpr int kTdMax = 8;
 struct McArgs {
   OpTable ops;
   int heff_w;  // host copy of ops.w[0], used to pick the kernel instance
+  int hreal;   // every off-diagonal entry of H_eff is real
   int stage_aux;      // set by the launcher: operators 1.. staged in shared memory
   int64_t aux_begin;  // first slot of operators 1.. (collapse, observables)
   int64_t aux_slots;  // number of slots of operators 1..

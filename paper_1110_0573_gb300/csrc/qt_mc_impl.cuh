@@ -188,7 +188,7 @@ struct GlobalStages {
   }
 };
 
-// Mixed register instances (W > 0): slot 0 of each row of H_eff is made its
+// Register instances (W > 0): slot 0 of each row of H_eff is made its
 // own-column slot, so that the right-hand side takes that product from the
 // thread's own state entry instead of the shared copy.  The host gives every
 // row of H_eff such a slot (the diagonal entry, or a zero padding entry).
@@ -211,6 +211,11 @@ template <typename T, int G, int R, int W, bool BLK, bool TD, bool GST = false>
 struct Traj {
   using V = typename CT<T>::V;
   static constexpr int WR = W > 0 ? W : 1;
+  // FP64 without time-dependent terms: the step in powers of H_eff (step()),
+  // its error as a squared norm.  (With them the FP64 kernel keeps the
+  // oracle's order of operations, stage by stage.)
+  static constexpr bool kPow = sizeof(T) == 8 && !TD;
+  static constexpr bool kOwn = sizeof(T) == 4 || kPow;  // slot 0 = own column
 
   const McArgs &a;
   const int lane;
@@ -225,6 +230,7 @@ struct Traj {
   const int *opoff;  // slot offset per operator relative to aval/acol
   int wh;            // ELL width of H_eff
   float inv2d;       // 1 / (2 d)
+  double inv2d_64;   // the same for the FP64 kernel
   T atol_t, rtol_t;  // tolerances in the kernel's precision
   V hv[R][WR];       // this lane's H_eff entries (W > 0)
   int hc[R][WR];
@@ -268,6 +274,7 @@ struct Traj {
     vlo = sizeof(T) == 4 ? reinterpret_cast<const V *>(a_.ops.val32lo) : nullptr;
     wh = opw[0];
     inv2d = 1.0f / (float)(2 * d);
+    inv2d_64 = sizeof(T) == 8 ? 1.0 / (double)(2 * d) : 0.0;
     atol_t = (T)a_.atol;
     rtol_t = (T)a_.rtol;
     if (W > 0) {
@@ -285,7 +292,7 @@ struct Traj {
             hc[q][s] = 0;
           }
         }
-        if constexpr (sizeof(T) == 4) {  // the own-column slot to slot 0
+        if constexpr (kOwn) {  // the own-column slot to slot 0
           int p = -1;
 #pragma unroll
           for (int s = WR - 1; s >= 0; --s)
@@ -583,8 +590,14 @@ struct Traj {
 #pragma unroll
         for (int s = 0; s < WR; ++s)  // mixed: padded slots hold 0 at column 0
           if (sizeof(T) == 4 || s < wh) {
-            // mixed: slot 0 is the row's own column (this thread's entry)
-            const V y = (sizeof(T) == 4 && s == 0) ? yq : yb[hc[q][s]];
+            // slot 0 is the row's own column (this thread's entry)
+            const V y = (kOwn && s == 0) ? yq : yb[hc[q][s]];
+            if constexpr (kPow) {
+              if (s > 0 && a.hreal) {  // FP64: real entries in two multiply-adds
+                acc.s = vfma(hv[q][s].x, y, acc.s);
+                continue;
+              }
+            }
             acc.mac(hv[q][s], y);
             if constexpr (kLo) acl.mac(hlo[row(q) * WR + s], y);
           }
@@ -738,7 +751,7 @@ struct Traj {
 
   // One Dormand-Prince step of length h from (psi, k[0] = f(psi)).  Writes the
   // 5th-order solution to ynew; with want_err evaluates k[6] = f(ynew) and
-  // returns the scaled RMS error norm, else returns 0.
+  // returns the scaled RMS error norm (kPow: its square), else returns 0.
   //
   // Mixed kernel: the stages use the FP32 entries of H_eff.  Their rounding
   // (relative 2^-24) is a fixed perturbation of the Hamiltonian whose effect
@@ -755,6 +768,57 @@ struct Traj {
     const T ht = h;
     n_rhs += want_err ? 6 : 5;
     V yt[R];
+    if constexpr (kPow) {
+      // The step in powers of the generator (DPP).  FP64-pipe bound: a warp
+      // issues an FP64 instruction every 65 cycles, and the stage sums,
+      // divisions, pow and sqrt were two thirds of its 480 per step
+      // (Jaynes-Cummings, dim 20).  500 trajectories 191 -> 89 ms.
+      // k[1], k[2]: the sums of the step and of the error; k[3]: v_(j+1).
+      double hp = ht;
+#pragma unroll
+      for (int q = 0; q < R; ++q) {
+        yt[q] = k[0][q];
+        k[1][q] = vmul(hp, yt[q]);
+        k[2][q] = vmul(DPP::e1 * hp, yt[q]);
+      }
+      auto power = [&](auto copy, int j, bool lead) {
+        rhs_f<false, decltype(copy)::value>(yt, k[3], u0, (T)0, 0, lead);
+        hp *= ht;
+        const double c = dpp_c(j) * hp, e = dpp_e(j) * hp;
+#pragma unroll
+        for (int q = 0; q < R; ++q) {
+          yt[q] = k[3][q];
+          k[1][q] = vfma(c, yt[q], k[1][q]);
+          if (want_err) k[2][q] = vfma(e, yt[q], k[2][q]);
+        }
+      };
+      const std::integral_constant<int, 0> c0;
+      const std::integral_constant<int, 1> c1;
+      power(c0, 2, !want_err);
+      power(c1, 3, false);
+      power(c0, 4, false);
+      power(c1, 5, false);
+      power(c0, 6, false);
+#pragma unroll
+      for (int q = 0; q < R; ++q) {
+        ynew[q] = vadd(psi[q], k[1][q]);
+        cnew[q] = cmake<V>(0.0, 0.0);
+      }
+      if (!want_err) return (T)0;
+      rhs_f<false, 1>(ynew, k[6], u0, (T)0, 0, false);
+      const double e7 = DPP::e7 * ht;
+      double sum = 0.0;
+#pragma unroll
+      for (int q = 0; q < R; ++q) {
+        if (row(q) >= d) continue;
+        const V er = vfma(e7, k[6][q], k[2][q]);
+        const double qx = er.x * recip(fma(rtol_t, max_abs(psi[q].x, ynew[q].x), atol_t));
+        const double qy = er.y * recip(fma(rtol_t, max_abs(psi[q].y, ynew[q].y), atol_t));
+        sum = fma(qx, qx, sum);
+        sum = fma(qy, qy, sum);
+      }
+      return gsum(sum) * inv2d_64;
+    }
     // stage input psi + h (c_1 k_1 + ... ): both components of each complex
     // entry with one packed multiply-add per coefficient
 #define QT_STAGE(EXPR)                                   \
@@ -851,10 +915,13 @@ struct Traj {
   }
 
   // Step-size controller in the scalar precision of the kernel: the FP64
-  // kernel uses the shared FP64 rule; the mixed kernel the same rule in FP32.
+  // kernel uses the shared FP64 rule (kPow: err is the squared norm); the mixed kernel
+  // the same rule in FP32.
   __device__ __forceinline__ T control(T h, T err, bool accepted, bool after_reject,
                                        bool clipped, T hprop) const {
-    if constexpr (sizeof(T) == 8) {
+    if constexpr (kPow) {
+      return dp_control_sq<double>(h, err, accepted, after_reject, clipped, hprop);
+    } else if constexpr (sizeof(T) == 8) {
       return dp_control(h, err, accepted, after_reject, clipped, hprop);
     } else {
       const float p = ex2_approx(-0.2f * lg2_approx(err));  // err^(-1/5)
@@ -1171,12 +1238,14 @@ struct Traj {
       int attempts = 0;
       while (u < L) {
         if (attempts++ >= a.max_steps) { set_status(a.status, QT_ESTEP); return false; }
-        const bool clipped = hprop >= L - u;
-        const T h = clipped ? L - u : hprop;
+        // (FP64: comparisons by integer order, off the FP64 pipe)
+        const T rest = L - u;
+        const bool clipped = kOff ? hprop >= rest : !pos_less((double)hprop, (double)rest);
+        const T h = clipped ? rest : hprop;
         if constexpr (kOff) {
           if (!clipped && h < hmin_off) { set_status(a.status, QT_ESTEP); return false; }
         } else {
-          if (!clipped && h < (T)dp_hmin((double)u, a.tlist[m])) {
+          if (!clipped && pos_less((double)h, 16.0 * 2.220446049250313e-16 * max_abs((double)u, (double)L))) {
             set_status(a.status, QT_ESTEP);
             return false;
           }
@@ -1184,8 +1253,8 @@ struct Traj {
         V ynew[R], cnew[R];
         float n2sum = 0.f;  // mixed: <ynew|ynew> in FP32, formed by step()
         const T err = step(psi, cps, k, u, h, ynew, cnew, true, &n2sum);
-        if (!isfinite(err)) { set_status(a.status, QT_ENUMERIC); return false; }
-        if (err > (T)1) {
+        if (!finite_bits(err)) { set_status(a.status, QT_ENUMERIC); return false; }
+        if (sizeof(T) == 8 ? pos_less(1.0, (double)err) : err > (T)1) {
           hprop = control(h, err, false, after_reject, clipped, hprop);
           after_reject = true;
           ++n_rej;
@@ -1200,7 +1269,7 @@ struct Traj {
         if (!below<sizeof(T) == 8>(ynew, cnew, rlo, rhi, n2, s32,
                                    sizeof(T) == 4 ? &n2sum : nullptr)) {
           if constexpr (sizeof(T) == 8) {
-            if (!isfinite(n2)) { set_status(a.status, QT_ENUMERIC); return false; }
+            if (!finite_bits(n2)) { set_status(a.status, QT_ENUMERIC); return false; }
             n2_cur = n2;
           } else {
             // a finite error norm implies a finite state; keep its FP32 norm
