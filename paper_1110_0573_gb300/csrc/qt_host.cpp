@@ -1945,7 +1945,7 @@ int qt_batch_config(qt_batch b, int *traj_block, int *small_group_dim, double *t
 struct qt_adjoint_s {
   int d = 0, nk = 0, n_seg = 0, batch = 0, maxs = 0;
   double t_seg = 0.0;
-  qt::OpTable ops;
+  qt::AdjArgs proto;  // the operators (qt_internal.h)
   std::vector<void *> dev;
   double2 *rho0 = nullptr, *ckpt = nullptr, *work = nullptr;
   int *nsteps = nullptr;
@@ -2002,9 +2002,7 @@ bool hermitian(const Csr &A) {
 }
 
 qt::AdjArgs adj_args(qt_adjoint a) {
-  qt::AdjArgs x;
-  std::memset(&x, 0, sizeof x);
-  x.ops = a->ops;
+  qt::AdjArgs x = a->proto;
   x.nk = a->nk;
   x.n_seg = a->n_seg;
   x.batch = a->batch;
@@ -2060,20 +2058,61 @@ int qt_adjoint_create(const qt_op *H0, const qt_op *Hd, const qt_op *A, int n_k,
   a->t_seg = t_seg;
   a->batch = batch;
   a->maxs = max_per_seg;
-  std::vector<int> cols, w;
-  std::vector<int64_t> off;
+  std::vector<int> cols;
   std::vector<double2> vals;
-  auto add = [&](const Csr &m) {
-    off.push_back((int64_t)cols.size());
-    w.push_back(ell_append(m, cols, vals));
+  std::memset(&a->proto, 0, sizeof a->proto);
+  qt::AdjArgs &op = a->proto;
+  // the stored entries of m (without its diagonal when off_diag)
+  auto add = [&](const Csr &m, bool off_diag) -> qt::AdjOp {
+    Csr x;
+    x.d = d;
+    x.ptr.assign(d + 1, 0);
+    qt::AdjOp o = {0, (int)cols.size(), 1};
+    for (int i = 0; i < d; ++i) {
+      for (int64_t p = m.ptr[i]; p < m.ptr[i + 1]; ++p) {
+        if (off_diag && m.col[p] == i) continue;
+        x.col.push_back(m.col[p]);
+        x.val.push_back(m.val[p]);
+        if (m.val[p].imag() != 0.0) o.real = 0;
+      }
+      x.ptr[i + 1] = (int64_t)x.col.size();
+    }
+    if (!x.col.empty()) o.w = ell_append(x, cols, vals);
+    return o;
   };
-  add(h0);
-  add(hd);
-  for (const Csr &m : Ak) add(m);
-  for (const Csr &m : Ak) add(csr_dagger(m));
-  for (const Csr &m : Ak) add(dagger_product(m));
-  add(p1);
-  add(p2);
+  auto diagonal = [](const Csr &m, int i) {
+    for (int64_t p = m.ptr[i]; p < m.ptr[i + 1]; ++p)
+      if (m.col[p] == i) return m.val[p];
+    return cplx(0.0, 0.0);
+  };
+  std::vector<double2> diag_h(d), diag_a((size_t)std::max(n_k, 1) * d, make_double2(0.0, 0.0));
+  std::vector<double> diag_n((size_t)std::max(n_k, 1) * d, 0.0);
+  op.op_h0 = add(h0, true);
+  op.op_hd = add(hd, true);
+  op.op_p1 = add(p1, false);
+  op.op_p2 = add(p2, false);
+  for (int i = 0; i < d; ++i) {
+    diag_h[i] = make_double2(diagonal(h0, i).real(), diagonal(hd, i).real());
+    if (diag_h[i].y != 0.0) op.hd_diag = 1;
+  }
+  for (int k = 0; k < n_k; ++k) {
+    bool diag = true;
+    for (int i = 0; i < d; ++i)
+      for (int64_t p = Ak[k].ptr[i]; p < Ak[k].ptr[i + 1]; ++p) diag = diag && Ak[k].col[p] == i;
+    const Csr nk = dagger_product(Ak[k]);
+    op.op_n[k] = add(nk, true);
+    for (int i = 0; i < d; ++i) diag_n[(size_t)k * d + i] = diagonal(nk, i).real();
+    if (diag) {
+      for (int i = 0; i < d; ++i) {
+        const cplx v = diagonal(Ak[k], i);
+        diag_a[(size_t)k * d + i] = make_double2(v.real(), v.imag());
+        if (v.imag() != 0.0) op.dk_complex = 1;
+      }
+    } else {
+      op.op_a[k] = add(Ak[k], false);
+      op.op_ad[k] = add(csr_dagger(Ak[k]), false);
+    }
+  }
   // rho0
   std::vector<double2> rho((size_t)d * d);
   if (state_is_ket) {
@@ -2088,6 +2127,14 @@ int qt_adjoint_create(const qt_op *H0, const qt_op *Hd, const qt_op *A, int n_k,
   } else {
     for (size_t q = 0; q < rho.size(); ++q) rho[q] = make_double2(state0[q].re, state0[q].im);
   }
+  // Hermitian up to rounding: the upper triangle determines every state
+  op.herm = 1;
+  for (int i = 0; i < d; ++i)
+    for (int j = i; j < d; ++j) {
+      const double2 u = rho[(size_t)i * d + j], v = rho[(size_t)j * d + i];
+      const double tol = 4e-16 * (std::abs(u.x) + std::abs(u.y));
+      if (!(std::abs(u.x - v.x) <= tol && std::abs(u.y + v.y) <= tol)) op.herm = 0;
+    }
   auto up = [&](const void *src, size_t bytes) -> void * {
     void *p = a->alloc(bytes);
     if (p && src && bytes && cudaMemcpy(p, src, bytes, cudaMemcpyHostToDevice) != cudaSuccess)
@@ -2096,14 +2143,12 @@ int qt_adjoint_create(const qt_op *H0, const qt_op *Hd, const qt_op *A, int n_k,
   };
   const int64_t n = (int64_t)d * d;
   a->slots = (int64_t)qt::adjoint_slots(max_per_seg);
-  a->ops.d = d;
-  a->ops.n_ops = (int)w.size();
-  a->ops.w = (int *)up(w.data(), w.size() * sizeof(int));
-  a->ops.off = (int64_t *)up(off.data(), off.size() * sizeof(int64_t));
-  a->ops.col = (int *)up(cols.data(), cols.size() * sizeof(int));
-  a->ops.val64 = (double2 *)up(vals.data(), vals.size() * sizeof(double2));
-  a->ops.val32 = nullptr;
-  a->ops.val32lo = nullptr;
+  op.ops.d = d;
+  op.ops.col = (int *)up(cols.data(), cols.size() * sizeof(int));
+  op.ops.val64 = (double2 *)up(vals.data(), vals.size() * sizeof(double2));
+  op.diag_h = (double2 *)up(diag_h.data(), diag_h.size() * sizeof(double2));
+  op.diag_a = (double2 *)up(diag_a.data(), diag_a.size() * sizeof(double2));
+  op.diag_n = (double *)up(diag_n.data(), diag_n.size() * sizeof(double));
   a->rho0 = (double2 *)up(rho.data(), rho.size() * sizeof(double2));
   a->nsteps = (int *)a->alloc((size_t)batch * n_seg * sizeof(int));
   a->hgrid = (double *)a->alloc((size_t)batch * n_seg * max_per_seg * sizeof(double));
@@ -2113,7 +2158,7 @@ int qt_adjoint_create(const qt_op *H0, const qt_op *Hd, const qt_op *A, int n_k,
   a->gamma = (double *)a->alloc((size_t)batch * std::max(n_k, 1) * sizeof(double));
   a->loss = (double *)a->alloc((size_t)batch * sizeof(double));
   a->ctl = (unsigned long long *)a->alloc(kCtlBytes);
-  if (!a->ops.w || !a->ops.off || !a->ops.col || !a->ops.val64 || !a->rho0 || !a->nsteps ||
+  if (!op.ops.col || !op.ops.val64 || !op.diag_h || !op.diag_a || !op.diag_n || !a->rho0 || !a->nsteps ||
       !a->hgrid || !a->ckpt || !a->work || !a->omega || !a->gamma || !a->loss || !a->ctl) {
     delete a;
     return fail(QT_ENOMEM, "device allocation of the adjoint workspace failed");

@@ -275,11 +275,25 @@ int batch_grid(int precision);
 size_t batch_ws_stride(int dmax, int precision);
 cudaError_t launch_batch_finalize(const BatchArgs &a, cudaStream_t s);
 
+// Stored entries of one operator of the adjoint kernels: ELL rows of width w
+// from slot off (w = 0: none); real: every value is real.
+struct AdjOp {
+  int w, off, real;
+};
+
 // Arguments of the master-equation adjoint kernels (one CTA per parameter
-// vector).  Operator table: 0 H0, 1 Hd, 2.. A_k, then A_k^dag, then
-// A_k^dag A_k, then P1, P2.
+// vector).  H0, Hd and N_k = A_k^dag A_k: off-diagonal entries, with their
+// diagonals apart; A_k and A_k^dag: all entries, or none when A_k is diagonal
+// (its entries are in diag_a then).
 struct AdjArgs {
   OpTable ops;
+  AdjOp op_h0, op_hd, op_p1, op_p2, op_a[8], op_ad[8], op_n[8];
+  const double2 *diag_h;  // [d]: diagonals of H0 and Hd
+  const double2 *diag_a;  // [nk][d]: A_k when diagonal, else zero
+  const double *diag_n;   // [nk][d]: diagonal of N_k
+  int hd_diag;            // Hd has diagonal entries
+  int dk_complex;         // a diagonal A_k has complex entries
+  int herm;               // rho0 is Hermitian: evaluate the upper triangle
   int nk, n_seg, batch, maxs;
   double t_seg;
   const double *omega;   // [batch][n_seg]
