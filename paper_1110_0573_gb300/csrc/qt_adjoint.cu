@@ -40,8 +40,7 @@
 // Transmon x cavity, dim 60, 256 drive vectors of 16 segments, forward and
 // backward: 571 -> 63 ms (before: every product complex and from the full
 // matrix, the stage sums of the tableau, 97 generator products and parameter
-// products per backward step where there are 17 now; FP64 pipe 90 % busy then,
-// 71 % of the floor of the instructions left now: 256 CTAs are 1.7 per SM).
+// products per backward step, the FP64 pipe 90 % busy).
 #include "qt_device.cuh"
 #include "qt_internal.h"
 

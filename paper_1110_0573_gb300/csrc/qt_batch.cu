@@ -84,7 +84,7 @@ __device__ void batch_mc_warp(const BatchArgs &a, const BatchProblem &P, const M
     }
     __syncwarp();
   }
-  Traj<T, G, R, W, false, false, false> tr(
+  Traj<T, G, R, W, false, kTdNone, false> tr(
       m, glane, mask, sm.ybuf[warp] + grp * (2 * G * R), val, val, P.ops.col, P.ops.w, P.opoff32,
       &sm.gs[warp][grp], hlo,
       sizeof(T) == 4 ? sm.lpb[warp] + grp * (2 * G * R) + glane : nullptr);

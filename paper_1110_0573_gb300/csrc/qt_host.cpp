@@ -1104,6 +1104,7 @@ int qt_mcsolve_dev(qt_system s, const qt_c128 *psi0_dev, const double *tlist_dev
   a.work = s->work();
   a.n_td = s->n_td;
   a.td_op0 = 1 + s->n_c + s->n_e;
+  a.td_w0 = s->n_td > 0 ? s->w_host[a.td_op0] : 0;
   a.td_off = s->td_off_dev;
   a.td_t = s->td_t_dev;
   a.td_v = s->td_v_dev;

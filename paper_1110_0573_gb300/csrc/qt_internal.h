@@ -58,6 +58,7 @@ struct McArgs {
   int *status;                   // first error code, 0 = ok
   unsigned long long *work;      // next trajectory to hand out
   int n_td, td_op0;              // time-dependent terms (0: none)
+  int td_w0;                     // ELL width of the first one
   const int64_t *td_off;
   const double *td_t, *td_v;
   void *stage_ws;                // dimensions above 2048: stage slabs, one per CTA
@@ -325,6 +326,7 @@ cudaError_t launch_mc_f64(const McArgs &a, cudaStream_t s);
 cudaError_t launch_mc_f32(const McArgs &a, cudaStream_t s);
 // the time-dependent and CTA-wide instances, compiled in their own units
 cudaError_t launch_mc_f32_td(const McArgs &a, int R, int W, cudaStream_t s);
+cudaError_t launch_mc_f32_td1(const McArgs &a, int R, int W, cudaStream_t s);
 cudaError_t launch_mc_f64_td(const McArgs &a, int R, int W, cudaStream_t s);
 cudaError_t launch_mc_f32_wide(const McArgs &a, cudaStream_t s);
 cudaError_t launch_mc_f32_dict(const McArgs &a, cudaStream_t s);

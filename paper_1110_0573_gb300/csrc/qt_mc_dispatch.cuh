@@ -46,7 +46,7 @@ cudaError_t dispatch_dict(const McArgs &a, cudaStream_t s) {
 template <typename T>
 cudaError_t dispatch_wide(const McArgs &a, cudaStream_t s) {
   const int d = a.ops.d;
-  if (d > 2048) return launch_inst<T, kBigG, kBigR, 0, true, false, true>(a, s);
+  if (d > 2048) return launch_inst<T, kBigG, kBigR, 0, true, kTdNone, true>(a, s);
   if (d > 1024) return launch_inst<T, 512, 4, 0, true>(a, s);
   return launch_inst<T, 256, 4, 0, true>(a, s);
 }
@@ -55,18 +55,38 @@ cudaError_t dispatch_wide(const McArgs &a, cudaStream_t s) {
 // its rows hold at most 4 entries, else read through the read-only cache.
 template <typename T>
 cudaError_t dispatch_td(const McArgs &a, int R, int W, cudaStream_t s) {
-  if (a.ops.d > 128) return launch_inst<T, 256, 4, 0, true, true>(a, s);
+  if (a.ops.d > 128) return launch_inst<T, 256, 4, 0, true, kTdAny>(a, s);
   if (R == 1) {
-    if (W == 4) return launch_inst<T, 32, 1, 4, false, true>(a, s);
-    return launch_inst<T, 32, 1, 0, false, true>(a, s);
+    if (W == 4) return launch_inst<T, 32, 1, 4, false, kTdAny>(a, s);
+    return launch_inst<T, 32, 1, 0, false, kTdAny>(a, s);
   }
   if (R == 2) {
-    if (W == 3) return launch_inst<T, 32, 2, 3, false, true>(a, s);
-    if (W == 4) return launch_inst<T, 32, 2, 4, false, true>(a, s);
-    return launch_inst<T, 32, 2, 0, false, true>(a, s);
+    if (W == 3) return launch_inst<T, 32, 2, 3, false, kTdAny>(a, s);
+    if (W == 4) return launch_inst<T, 32, 2, 4, false, kTdAny>(a, s);
+    return launch_inst<T, 32, 2, 0, false, kTdAny>(a, s);
   }
-  if (W == 4) return launch_inst<T, 32, 4, 4, false, true>(a, s);
-  return launch_inst<T, 32, 4, 0, false, true>(a, s);
+  if (W == 4) return launch_inst<T, 32, 4, 4, false, kTdAny>(a, s);
+  return launch_inst<T, 32, 4, 0, false, kTdAny>(a, s);
+}
+
+// One time-dependent term of at most two entries per row, H_eff in registers
+// (mixed precision, its own unit qt_mc_f32_td1.cu).  The general instances
+// carry the loop over terms, the read-only-cache products and a piece look-up
+// in every inlined stage, and were bound by instruction fetch (no_instruction
+// 4.5 stalls per issue); these hold one term's two entries in registers and
+// look pieces up once per step.  Kerr cavity with a ramped drive, dim 64, 16384
+// trajectories: 104.4 -> 38.5 ms (three CTAs per SM; four, at 128 registers,
+// spill: 39.1 ms, and 4.2 against 3.8 ms for 1000 trajectories).
+inline bool use_td_one(const McArgs &a, int W) {
+  return a.n_td == 1 && a.td_w0 <= 2 && a.ops.d <= 128 && (W == 3 || W == 4);
+}
+
+template <typename T>
+cudaError_t dispatch_td_one(const McArgs &a, int R, int W, cudaStream_t s) {
+  if (R == 1) return launch_inst<T, 32, 1, 4, false, kTdOne>(a, s);
+  if (R == 2 && W == 3) return launch_inst<T, 32, 2, 3, false, kTdOne>(a, s);
+  if (R == 2) return launch_inst<T, 32, 2, 4, false, kTdOne>(a, s);
+  return launch_inst<T, 32, 4, 4, false, kTdOne>(a, s);
 }
 
 // Time-independent warp groups (dimension <= 128).

@@ -10,7 +10,8 @@ cudaError_t launch_mc_f32(const McArgs &a, cudaStream_t s) {
   choose(a.ops.d, a.heff_w, R, W);
   switch (mc_unit(a)) {
     case McUnit::kWide: return use_dict(a) ? launch_mc_f32_dict(a, s) : launch_mc_f32_wide(a, s);
-    case McUnit::kTd: return launch_mc_f32_td(a, R, W, s);
+    case McUnit::kTd:
+      return use_td_one(a, W) ? launch_mc_f32_td1(a, R, W, s) : launch_mc_f32_td(a, R, W, s);
     default: return dispatch_warp<float>(a, R, W, s);
   }
 }

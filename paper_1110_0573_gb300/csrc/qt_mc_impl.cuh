@@ -92,6 +92,41 @@ __device__ __noinline__ TdPiece<T> td_lookup_piece(const double *kt, const doubl
   return p;
 }
 
+// f_0 at the stage offsets s[0..5] of a step that leaves the cached piece p
+// (times from tb): each from the piece in use when it lies in it, else from the
+// piece around it, which becomes the one in use.  Out of line, once per step.
+template <typename T>
+struct TdStep {
+  T f[6], p[4];
+};
+
+template <typename T>
+__device__ __noinline__ TdStep<T> td_step_coefs(const double *kt, const double *kv, int64_t a0,
+                                                int64_t b0, double tb, T u0, T h, T p_0, T p_1,
+                                                T p_2, T p_3) {
+  TdStep<T> r;
+  r.p[0] = p_0;
+  r.p[1] = p_1;
+  r.p[2] = p_2;
+  r.p[3] = p_3;
+  const T c[4] = {(T)DP::c2, (T)DP::c3, (T)DP::c4, (T)DP::c5};
+#pragma unroll
+  for (int i = 0; i < 6; ++i) {
+    const T s = i < 4 ? tfma(c[i], h, u0) : u0 + h;
+    if (!(s >= r.p[2] && s <= r.p[3])) {
+      const TdPiece<T> q = td_lookup_piece<T>(kt, kv, a0, b0, tb, s);
+      r.p[0] = q.f0;
+      r.p[1] = q.slope;
+      r.p[2] = q.lo;
+      r.p[3] = q.hi;
+      r.f[i] = q.f;
+    } else {
+      r.f[i] = tfma(r.p[1], s, r.p[0]);
+    }
+  }
+  return r;
+}
+
 // FP64 scalars of one group's current trajectory.
 struct GroupScalars {
   double r;                 // pending jump threshold
@@ -207,7 +242,12 @@ __host__ __device__ constexpr int heff_swapped_slot(int sl, int p) {
   return p <= 0 ? sl : (sl == 0 ? p : (sl == p ? 0 : sl));
 }
 
-template <typename T, int G, int R, int W, bool BLK, bool TD, bool GST = false>
+// Time-dependent terms of an instance (template TD): none; exactly one whose
+// rows hold at most two entries (a ladder drive a + a^dag, a spin's sigma_x),
+// in registers and with none of the general code; any.
+constexpr int kTdNone = 0, kTdOne = 1, kTdAny = 2;
+
+template <typename T, int G, int R, int W, bool BLK, int TD, bool GST = false>
 struct Traj {
   using V = typename CT<T>::V;
   static constexpr int WR = W > 0 ? W : 1;
@@ -250,7 +290,7 @@ struct Traj {
   // the first time-dependent term: its ELL rows in registers when at most 4
   // wide (tw0 >= 0), and its current linear piece {f at offset 0, slope,
   // first offset, last offset} (every thread of the group holds the same)
-  static constexpr int TR = (TD && W > 0) ? 4 : 1;
+  static constexpr int TR = TD == kTdOne ? 2 : (TD && W > 0) ? 4 : 1;
   V tv[R][TR];
   int tc[R][TR];
   int tw0 = -1;
@@ -619,7 +659,17 @@ struct Traj {
       k[q].y = -hy.x;
     }
     }
-    if constexpr (TD) {
+    if constexpr (TD == kTdOne) {
+#pragma unroll
+      for (int q = 0; q < R; ++q) {
+        CAcc<V> acd;
+#pragma unroll
+        for (int s = 0; s < TR; ++s) acd.mac(tv[q][s], yb[tc[q][s]]);
+        const V hy = acd.get();
+        k[q].x = tfma(f0, hy.y, k[q].x);
+        k[q].y = tfma(-f0, hy.x, k[q].y);
+      }
+    } else if constexpr (TD != kTdNone) {
       for (int t = 0; t < a.n_td; ++t) {
         const T f = t == 0 ? f0 : td_coef(t, ts);
 #pragma unroll
@@ -832,9 +882,22 @@ struct Traj {
     // the cached piece when the whole step lies in it
     bool fast = true;
     if constexpr (TD) fast = sizeof(T) == 4 && u0 >= p0[2] && u0 + ht <= p0[3];
+    TdStep<T> tds;
+    if constexpr (TD == kTdOne) {
+      if (!fast) {
+        tds = td_step_coefs<T>(a.td_t, a.td_v, a.td_off[0], a.td_off[1] - 1, gs->tb, u0, ht, p0[0],
+                               p0[1], p0[2], p0[3]);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) p0[i] = tds.p[i];
+      }
+    }
+    int stage = 0;
     auto coef = [&](T so) -> T {
       if constexpr (!TD) {
         return (T)0;
+      } else if constexpr (TD == kTdOne) {
+        const int i = stage++;
+        return fast ? tfma(p0[1], so, p0[0]) : tds.f[i];
       } else {
         if (a.n_td == 0) return (T)0;
         return fast ? tfma(p0[1], so, p0[0]) : td_coef(0, so);
@@ -1428,13 +1491,13 @@ __host__ __device__ constexpr int mc_block() {
 // instances fit 128 registers (16 warps per SM; 168 and 12 warps with the
 // time-dependent terms); the FP64 and wide instances keep up to 255 registers
 // rather than spill; a CTA-wide group runs one CTA.
-template <typename T, int G, int R, int W, bool BLK, bool TD>
+template <typename T, int G, int R, int W, bool BLK, int TD>
 __host__ __device__ constexpr int mc_min_blocks() {
   return BLK ? ((W < 0 && G == 256) ? 2 : 1)
              : ((sizeof(T) == 4 && R <= 2 && W <= 4) ? (TD ? 3 : 4) : 2);
 }
 
-template <typename T, int G, int R, int W, bool BLK, bool TD, bool GST>
+template <typename T, int G, int R, int W, bool BLK, int TD, bool GST>
 __global__ void __launch_bounds__((mc_block<G, BLK>()), (mc_min_blocks<T, G, R, W, BLK, TD>()))
     mc_kernel(const __grid_constant__ McArgs a) {
   using V = typename CT<T>::V;
@@ -1529,7 +1592,7 @@ __global__ void __launch_bounds__((mc_block<G, BLK>()), (mc_min_blocks<T, G, R, 
   }
 }
 
-template <typename T, int G, int R, int W, bool BLK, bool TD = false, bool GST = false>
+template <typename T, int G, int R, int W, bool BLK, int TD = kTdNone, bool GST = false>
 cudaError_t launch_inst(const McArgs &a_in, cudaStream_t s) {
   using V = typename CT<T>::V;
   auto kern = mc_kernel<T, G, R, W, BLK, TD, GST>;

@@ -45,8 +45,8 @@ def test_gradients(qt, form, d):
         A = [rand(d, rng, False, cplx), sp.diags(np.exp(1j * np.arange(d))).tocsr()]
     if form == "no_rates":
         A = []
-    if form == "many_steps":  # about 60 steps a segment
-        H0, maxs = 40.0 * H0 + 60.0 * S.num(d), 256
+    if form == "many_steps":  # up to 2400 steps a segment at d = 17
+        H0, maxs = 40.0 * H0 + 60.0 * S.num(d), 4096
     P1, P2 = rand(d, rng, True), rand(d, rng, True)
     psi = rng.standard_normal(d) + 1j * rng.standard_normal(d)
     if form == "not_hermitian":
