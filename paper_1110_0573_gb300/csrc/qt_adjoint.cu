@@ -651,9 +651,13 @@ __global__ void __launch_bounds__(kAdjBlock, 1) adjoint_backward_kernel(const __
   }
 }
 
+// The kernels' limit is that of the largest problem (dim 64, 8 decay rates),
+// whatever this one takes: it belongs to the process, and one set for a
+// smaller problem on another thread would refuse this thread's launch.
 cudaError_t smem_for(const void *kern, const AdjArgs &a, size_t *bytes) {
   *bytes = adj_smem(a.ops.d, a.nk).total;
-  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)*bytes);
+  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)adj_smem(64, 8).total);
 }
 
 }  // namespace

@@ -144,6 +144,17 @@ SmallMode small_mode(const MeArgs &a, int precision, size_t *smem) {
   return SmallMode::kWork;
 }
 
+static_assert(sizeof(MeArgs) <= 1024, "static shared memory beside kSmallSmemMax");
+
+// The limit of every instance with dynamic shared memory (one value for all
+// sizes: see kSmallSmemMax).
+template <typename K>
+cudaError_t set_smem_limit(K kern, size_t smem) {
+  if (smem == 0) return cudaSuccess;
+  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)kSmallSmemMax);
+}
+
 // Resident CTAs of a kernel with smem bytes of dynamic shared memory, at most
 // units (negative on error).
 template <typename K>
@@ -151,9 +162,7 @@ int block_grid(K kern, size_t smem, int64_t units) {
   int dev = 0, sms = 0, per_sm = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return -1;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return -1;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-      cudaSuccess)
-    return -1;
+  if (set_smem_limit(kern, smem) != cudaSuccess) return -1;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kMeBlock, smem) != cudaSuccess)
     return -1;
   if (per_sm < 1) return -1;
@@ -196,8 +205,7 @@ cudaError_t launch_corr_block(const MeArgs &a, const CorrArgs &c, int grid, int 
   size_t smem;
   const SmallMode m = small_mode(a, precision, &smem);
   return with_corr_kernel(precision, m, [&](auto *k) {
-    cudaError_t e =
-        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = set_smem_limit(k, smem);
     if (e != cudaSuccess) return e;
     k<<<grid, kMeBlock, smem, s>>>(a, c);
     return cudaGetLastError();
@@ -215,8 +223,7 @@ cudaError_t launch_prop_block(const MeArgs &a, const PropArgs &p, int grid, int 
   size_t smem;
   const SmallMode m = small_mode(a, precision, &smem);
   return with_prop_kernel(precision, m, [&](auto *k) {
-    cudaError_t e =
-        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = set_smem_limit(k, smem);
     if (e != cudaSuccess) return e;
     k<<<grid, kMeBlock, smem, s>>>(a, p);
     return cudaGetLastError();

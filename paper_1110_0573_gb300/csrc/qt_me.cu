@@ -132,7 +132,8 @@ namespace {
 template <typename T, bool CL, bool KS>
 cudaError_t launch_small_inst(const MeArgs &a, size_t smem, int ranks, cudaStream_t s) {
   cudaError_t e = cudaFuncSetAttribute(me_small_kernel<T, CL, KS>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)kSmallSmemMax);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(ranks);
