@@ -591,7 +591,12 @@ int qt_adjoint_destroy(qt_adjoint a);
  * as output times); keeps each vector's accepted step lengths (the frozen
  * grid), rho at the segment ends and a copy of the parameters for the
  * backward pass.  omega_dev[batch * n_seg], gamma_dev[batch * n_k],
- * loss_dev[batch]: device pointers.  Asynchronous on stream. */
+ * loss_dev[batch]: device pointers.  Asynchronous on stream.  A vector whose
+ * solve ends early (QT_ESTEP: more than max_per_seg steps in a segment, or a
+ * step limit; QT_ENUMERIC) sets the status in stats_dev and has the loss NaN,
+ * as it has in qt_adjoint_loss_fixed_dev and its gradients in
+ * qt_adjoint_backward_dev; its grid ends with the last completed segment
+ * (nsteps 0 from there on).  The other vectors are not affected. */
 int qt_adjoint_forward_dev(qt_adjoint a, const double *omega_dev, const double *gamma_dev,
                            const qt_opts *o, double *loss_dev, qt_stats *stats_dev,
                            void *stream);

@@ -51,6 +51,7 @@ namespace {
 constexpr int kAdjBlock = 512;
 
 __device__ __forceinline__ double2 cj(double2 v) { return make_double2(v.x, -v.y); }
+__device__ __forceinline__ double nan_value() { return __longlong_as_double(0x7ff8000000000000ll); }
 
 struct AdjCtl {
   double h;
@@ -250,6 +251,11 @@ struct Adj {
     }
     return acc;
   }
+  // The last forward pass of this vector did not reach the final time: its
+  // grid and checkpoints end before.
+  __device__ bool failed() const {
+    return a.nsteps[(int64_t)blockIdx.x * a.n_seg + a.n_seg - 1] == 0;
+  }
   // c_k h^k and e_k h^k by lanes 0..7 of warp 0.
   __device__ __forceinline__ void powers(double h) const {
     if (threadIdx.x < 8) {
@@ -263,6 +269,10 @@ struct Adj {
 
 // Forward solve of one parameter vector: adaptive (recording the grid and
 // the segment checkpoints) or on the recorded grid (a.fixed, loss only).
+// nsteps[s] stays 0 for a segment that was not completed (an error status), so
+// a vector's grid is whole exactly when that of its last segment is not 0:
+// Adj::failed() tells the passes on the recorded grid, which return NaN then
+// (as does the loss of the failing pass itself).
 __global__ void __launch_bounds__(kAdjBlock, 1) adjoint_forward_kernel(const __grid_constant__ AdjArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
   Adj A(a, smem);
@@ -277,6 +287,12 @@ __global__ void __launch_bounds__(kAdjBlock, 1) adjoint_forward_kernel(const __g
   double2 *y0 = A.y0, *y1 = A.y1;
   AdjCtl *ctl = A.ctl;
   const bool lead = threadIdx.x < 32;
+  if (a.fixed && A.failed()) {
+    if (threadIdx.x == 0) a.loss[b] = nan_value();
+    return;
+  }
+  if (!a.fixed)
+    for (int s = threadIdx.x; s < a.n_seg; s += kAdjBlock) nsteps[s] = 0;
   auto checkpoint = [&](int s) {
     for (int x = threadIdx.x; x < n; x += kAdjBlock) ckpt[(int64_t)s * n + x] = y1[x / d * ld + x % d];
   };
@@ -474,7 +490,7 @@ __global__ void __launch_bounds__(kAdjBlock, 1) adjoint_forward_kernel(const __g
   A.reduce(v, 1);
   if (threadIdx.x == 0) {
     if (status != QT_OK) set_status(a.status, status);
-    a.loss[b] = v[0];
+    a.loss[b] = status == QT_OK ? v[0] : nan_value();
     atomicAdd(a.counters + 0, n_acc);
     atomicAdd(a.counters + 1, n_rej);
     atomicAdd(a.counters + 2, n_rhs);
@@ -495,6 +511,11 @@ __global__ void __launch_bounds__(kAdjBlock, 1) adjoint_backward_kernel(const __
   AdjCtl *ctl = A.ctl;
   double *gk = A.gk;
   const double scale = a.dloss ? a.dloss[b] : 1.0;
+  if (A.failed()) {
+    for (int s = threadIdx.x; s < a.n_seg; s += kAdjBlock) a.g_omega[(int64_t)b * a.n_seg + s] = nan_value();
+    for (int k = threadIdx.x; k < nk; k += kAdjBlock) a.g_gamma[(int64_t)b * nk + k] = nan_value();
+    return;
+  }
   // workspace: lambda, D, P2, the sums of conj(a) v, a step sum, v_1..v_5 of
   // one recomputed step, the segment's states, then v_1..v_5 of its first
   // `kept` steps

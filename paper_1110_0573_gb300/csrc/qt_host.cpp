@@ -2151,7 +2151,8 @@ int qt_adjoint_create(const qt_op *H0, const qt_op *Hd, const qt_op *A, int n_k,
   op.diag_a = (double2 *)up(diag_a.data(), diag_a.size() * sizeof(double2));
   op.diag_n = (double *)up(diag_n.data(), diag_n.size() * sizeof(double));
   a->rho0 = (double2 *)up(rho.data(), rho.size() * sizeof(double2));
-  a->nsteps = (int *)a->alloc((size_t)batch * n_seg * sizeof(int));
+  const std::vector<int> none((size_t)batch * n_seg, 0);  // no forward pass yet
+  a->nsteps = (int *)up(none.data(), none.size() * sizeof(int));
   a->hgrid = (double *)a->alloc((size_t)batch * n_seg * max_per_seg * sizeof(double));
   a->ckpt = (double2 *)a->alloc((size_t)batch * (n_seg + 1) * n * sizeof(double2));
   a->work = (double2 *)a->alloc((size_t)batch * a->slots * n * sizeof(double2));

@@ -303,7 +303,7 @@ struct AdjArgs {
   double rtol, atol;
   int64_t max_steps;
   int fixed;             // 1: integrate on the recorded grid, loss only
-  int *nsteps;           // [batch][n_seg]
+  int *nsteps;           // [batch][n_seg], 0 for a segment not completed
   double *hgrid;         // [batch][n_seg][maxs]
   double2 *ckpt;         // [batch][n_seg + 1][d*d]
   double2 *work;         // [batch][slots][d*d]

@@ -620,7 +620,9 @@ def master_equation_loss(adjoint, omega, gamma, opts):
     problem: forward by the adaptive solver, backward by the library's
     adjoint kernel on the forward pass's step grid (segment checkpoints
     recomputed).  omega: float64 CUDA tensor [batch, n_seg]; gamma:
-    [batch, n_k]."""
+    [batch, n_k].  A vector that its forward pass could not finish (more than
+    max_per_seg steps in a segment, or a non-finite parameter) has NaN loss
+    and gradients."""
     import torch
 
     class _MasterEquationLoss(torch.autograd.Function):
