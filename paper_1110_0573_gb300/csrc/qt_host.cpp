@@ -1446,6 +1446,7 @@ int qt_propagator_dev(qt_system s, const double *tlist_dev, int n_t, const qt_op
   me_args(s, &o2, 1, s->aux, a);
   a.n_t = n_t;
   a.tlist = tlist_dev;
+  a.n_e = 0;  // no expectation values, whatever observables the system holds
   a.expect = nullptr;
   a.states = nullptr;
   a.state_is_ket = 0;
