@@ -638,8 +638,11 @@ int me_setup(qt_system s, const qt_opts *o, bool is_ket, qt::MeArgs &a) {
   const bool small_herm = small && is_ket && o->me_method == QT_ME_AUTO;
   size_t ws = qt::me_workspace_bytes(s->d, o->precision, grid);
   if (small) {
+    // for all entries, whichever this solve evaluates: the forms of one system
+    // share a workspace, and a solve that follows another one (perhaps captured
+    // in a graph) neither frees nor allocates
     me_args(s, o, grid, nullptr, a);
-    ws = std::max(ws, qt::small_workspace_bytes(a, o->precision, small_herm, true));
+    ws = std::max(ws, qt::small_workspace_bytes(a, o->precision, false, true));
   }
   if ((rc = ensure_ws(s, ws))) return rc;
   me_args(s, o, grid, s->ws, a);
