@@ -1282,8 +1282,7 @@ int qt_steadystate_dev(qt_system s, double tol, int64_t max_iter, int krylov_dim
   int m = krylov_dim > 0 ? krylov_dim : 600;
   if (m > 4096) return fail(QT_EINVAL, "krylov_dim must be <= 4096");
   // the grid: every resident CTA; each owns a chunk of the d*d entries held
-  // in shared memory (at most 200 KB per CTA)
-  constexpr size_t kSmemMax = 200 * 1024;
+  // in shared memory
   int grid = qt::gmres_grid(0);
   if (grid <= 0) return fail(QT_ECUDA, "cannot size the cooperative launch");
   int chunk = 0;
@@ -1291,7 +1290,7 @@ int qt_steadystate_dev(qt_system s, double tol, int64_t max_iter, int krylov_dim
   for (int pass = 0; pass < 2; ++pass) {
     chunk = (int)((n + grid - 1) / grid);
     smem = qt::gmres_smem_bytes(chunk, m);
-    if (smem > kSmemMax)
+    if (smem > qt::kGmresSmemMax)
       return fail(QT_ENOTIMPL,
                   "dim %d with krylov_dim %d needs %zu bytes of shared memory per CTA; use a "
                   "smaller krylov_dim or qt_propagator_steadystate",

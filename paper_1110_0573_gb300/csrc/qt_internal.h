@@ -10,6 +10,13 @@
 
 namespace qt {
 
+// Dynamic shared memory.  The limit that cudaFuncSetAttribute sets belongs to
+// the kernel and the process, not to a launch: every caller of a kernel sets
+// one value, that of the largest launch it may have.  With the size of each
+// launch, a smaller one on another thread would refuse this thread's.
+constexpr size_t kSmemPerCta = 227 * 1024;    // static and dynamic, at most
+constexpr size_t kGmresSmemMax = 200 * 1024;  // of the GMRES kernel (9 KB static beside it)
+
 // Operators on the device are stored in ELLPACK form, slot-major: the s-th
 // stored entry of row i sits at off + s * d + i (consecutive rows of one slot
 // are contiguous, so threads that own consecutive rows load coalesced).

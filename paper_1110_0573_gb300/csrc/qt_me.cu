@@ -84,15 +84,21 @@ size_t dyn_bytes(int n_cslots, int n_cterms) {
   return herm_smem_bytes<typename CT<T>::V>(n_cslots, n_cterms);
 }
 
+// The limit of me_kernel: the Hermitian solver with the most collapse operators
+// that it stages (one value for all launches: see kSmemPerCta).
+template <typename T>
+cudaError_t set_me_limit() {
+  return cudaFuncSetAttribute(me_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)dyn_bytes<T>(kCSlotsMax, kCTermsMax));
+}
+
 template <typename T>
 int grid_for(int d, bool herm, int n_cslots, int n_cterms) {
   int dev = 0, sms = 0, per_sm = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return -1;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return -1;
   const size_t dyn = herm ? dyn_bytes<T>(n_cslots, n_cterms) : 0;
-  if (cudaFuncSetAttribute(me_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) !=
-      cudaSuccess)
-    return -1;
+  if (set_me_limit<T>() != cudaSuccess) return -1;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, me_kernel<T>, kMeBlock, dyn) !=
       cudaSuccess)
     return -1;
@@ -176,8 +182,7 @@ cudaError_t launch_me_t(const MeArgs &a, cudaStream_t s) {
     return cudaGetLastError();
   }
   const size_t dyn = a.herm ? dyn_bytes<T>(a.n_cslots, a.n_cterms) : 0;
-  cudaError_t e =
-      cudaFuncSetAttribute(me_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
+  const cudaError_t e = set_me_limit<T>();
   if (e != cudaSuccess) return e;
   void *args[] = {const_cast<MeArgs *>(&a)};
   return cudaLaunchCooperativeKernel((const void *)me_kernel<T>, dim3(a.grid), dim3(kMeBlock),

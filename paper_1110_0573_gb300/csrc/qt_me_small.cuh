@@ -89,11 +89,9 @@ __device__ __forceinline__ void smac(float4 c, float2 x, float2 &out, float2 &lo
 
 constexpr int kSmallMaxRanks = 8;
 // Dynamic shared memory of one CTA: the 227 KB that a CTA may have, less 1 KB
-// for the static variables of the kernels that call the solver.  Every launch
-// sets the kernels' limit to this value and not to its own size: the limit
-// belongs to the process, so that of a smaller solve on another thread would
-// refuse this thread's launch.
-constexpr size_t kSmallSmemMax = 226 * 1024;
+// for the static variables of the kernels that call the solver; the limit of
+// every launch, whatever its size (see kSmemPerCta).
+constexpr size_t kSmallSmemMax = kSmemPerCta - 1024;
 
 // What warp 0 of each CTA hands to the others after each step attempt.
 struct SmallCtl {

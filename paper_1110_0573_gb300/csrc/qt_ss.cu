@@ -479,8 +479,8 @@ int gmres_grid(size_t smem) {
   int dev = 0, sms = 0, per_sm = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return -1;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return -1;
-  if (cudaFuncSetAttribute(gmres_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-      cudaSuccess)
+  if (cudaFuncSetAttribute(gmres_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)kGmresSmemMax) != cudaSuccess)
     return -1;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, gmres_kernel, kGmBlock, smem) !=
       cudaSuccess)
@@ -491,8 +491,8 @@ int gmres_grid(size_t smem) {
 
 cudaError_t launch_gmres(const MeArgs &a, const GmArgs &g, int grid, size_t smem,
                          cudaStream_t s) {
-  cudaError_t e =
-      cudaFuncSetAttribute(gmres_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = cudaFuncSetAttribute(gmres_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)kGmresSmemMax);
   if (e != cudaSuccess) return e;
   void *args[] = {const_cast<MeArgs *>(&a), const_cast<GmArgs *>(&g)};
   return cudaLaunchCooperativeKernel((const void *)gmres_kernel, dim3(grid), dim3(kGmBlock), args,
