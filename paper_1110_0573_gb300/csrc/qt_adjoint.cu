@@ -434,8 +434,8 @@ __global__ void __launch_bounds__(kAdjBlock, 1) adjoint_forward_kernel(const __g
           if (!a.fixed) {
             const double2 er = vfma(e7, g, err[e]);
             const double2 r = rho[e], yn = y1[i * ld + j];
-            const double qx = er.x * recip(fma(a.rtol, max_abs(r.x, yn.x), a.atol));
-            const double qy = er.y * recip(fma(a.rtol, max_abs(r.y, yn.y), a.atol));
+            const double qx = ratio(er.x, fma(a.rtol, max_abs(r.x, yn.x), a.atol));
+            const double qy = ratio(er.y, fma(a.rtol, max_abs(r.y, yn.y), a.atol));
             acc = fma(A.weight(i, j), fma(qx, qx, qy * qy), acc);
           }
           err[e] = g;

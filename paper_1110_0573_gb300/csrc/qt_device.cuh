@@ -242,19 +242,26 @@ __device__ __forceinline__ double dp_control(double h, double err, bool accepted
   return h * fmax(0.2, 0.9 * pow(err, -0.2));
 }
 
-// 1 / x.  FP64: one third-order Householder step from the hardware's
-// approximate reciprocal (about 20 bits), three multiply-adds, within an ulp
-// or two; numbers whose reciprocal or approximation leaves the normal range
-// are divided.  An FP64 division costs about three times as many FP64
-// instructions, and those bound the FP64 solvers.
-__device__ __forceinline__ float recip(float x) { return rcp_approx(x); }
-__device__ __forceinline__ double recip(double x) {
-  const int hi = __double2hiint(x) & 0x7fffffff;
-  if (hi < 0x01000000 || hi >= 0x7e000000) return 1.0 / x;  // 2^-1007 .. 2^993
+// x / w for an error weight w >= 0.  FP64: the product with 1 / w by one
+// third-order Householder step from the hardware's approximate reciprocal
+// (about 20 bits), three multiply-adds, within 2 ulp of the quotient; an FP64
+// division costs about three times as many FP64 instructions, and those bound
+// the FP64 solvers.  FP32: the product with the approximate reciprocal, within
+// 2^-22.  Weights whose reciprocal or its approximation leaves the normal range
+// (2^-1007 .. 2^993, 2^-126 .. 2^126) are divided: with atol = 0 they belong to
+// entries of a state that are as small.
+__device__ __forceinline__ double ratio(double x, double w) {
+  const int hi = __double2hiint(w);
+  if (hi < 0x01000000 || hi >= 0x7e000000) return x / w;
   double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  const double e = fma(-x, y, 1.0);
-  return fma(y, fma(e, e, e), y);
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(w));
+  const double e = fma(-w, y, 1.0);
+  return x * fma(y, fma(e, e, e), y);
+}
+__device__ __forceinline__ float ratio(float x, float w) {
+  const int b = __float_as_int(w);
+  if (b < 0x00800000 || b >= 0x7e800000) return x / w;
+  return x * rcp_approx(w);
 }
 
 // x^(-1/10) for x in [1e-30, 1e30] from an FP32 value with relative error e:

@@ -862,8 +862,8 @@ struct Traj {
       for (int q = 0; q < R; ++q) {
         if (row(q) >= d) continue;
         const V er = vfma(e7, k[6][q], k[2][q]);
-        const double qx = er.x * recip(fma(rtol_t, max_abs(psi[q].x, ynew[q].x), atol_t));
-        const double qy = er.y * recip(fma(rtol_t, max_abs(psi[q].y, ynew[q].y), atol_t));
+        const double qx = ratio(er.x, fma(rtol_t, max_abs(psi[q].x, ynew[q].x), atol_t));
+        const double qy = ratio(er.y, fma(rtol_t, max_abs(psi[q].y, ynew[q].y), atol_t));
         sum = fma(qx, qx, sum);
         sum = fma(qy, qy, sum);
       }

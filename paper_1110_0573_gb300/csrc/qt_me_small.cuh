@@ -606,8 +606,8 @@ struct SmallSolver {
           const V er = vfma(ce, g, err[l]);
           err[l] = g;
           const V r = rho[l], yn = y1[i * ld + j];
-          const T qx = er.x * recip(tfma(rt, max_abs(r.x, yn.x), at));
-          const T qy = er.y * recip(tfma(rt, max_abs(r.y, yn.y), at));
+          const T qx = ratio(er.x, tfma(rt, max_abs(r.x, yn.x), at));
+          const T qy = ratio(er.y, tfma(rt, max_abs(r.y, yn.y), at));
           const T q2 = tfma(qx, qx, qy * qy);
           acc += herm && i != j ? (T)2 * q2 : q2;
         });
