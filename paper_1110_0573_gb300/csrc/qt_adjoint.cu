@@ -41,6 +41,8 @@
 // backward: 571 -> 63 ms (before: every product complex and from the full
 // matrix, the stage sums of the tableau, 97 generator products and parameter
 // products per backward step, the FP64 pipe 90 % busy).
+#include <type_traits>
+
 #include "qt_device.cuh"
 #include "qt_internal.h"
 
@@ -55,7 +57,10 @@ __device__ __forceinline__ double nan_value() { return __longlong_as_double(0x7f
 
 struct AdjCtl {
   double h;
-  double c[8], e[8];  // c_k h^k, e_k h^k (e_7: h alone)
+  // the weights of F v_(k-1) and Tr(P2 v_(k-1)), c_k h^k, those of the error, e_k h^k
+  // (e_7: h alone), and those of lambda in a_k, c_k h^k; for a step that is
+  // dpp_scaled c_k h, e_k h and c_k
+  double c[8], e[8], l[8];
   int accepted, done, status;
 };
 
@@ -251,18 +256,25 @@ struct Adj {
     }
     return acc;
   }
+  // This thread's entries of m by h (a step that is dpp_scaled).
+  __device__ void scale(double2 *m, double h) const {
+    each([&](int, int i, int j) { put(m, i, j, vmul(h, m[i * ld + j])); });
+  }
   // The last forward pass of this vector did not reach the final time: its
   // grid and checkpoints end before.
   __device__ bool failed() const {
     return a.nsteps[(int64_t)blockIdx.x * a.n_seg + a.n_seg - 1] == 0;
   }
-  // c_k h^k and e_k h^k by lanes 0..7 of warp 0.
+  // The coefficients of a step of length h by lanes 0..7 of warp 0.
   __device__ __forceinline__ void powers(double h) const {
     if (threadIdx.x < 8) {
+      const bool scaled = dpp_scaled(h);
       double p = 1.0;
-      for (int q = 0; q < (int)threadIdx.x; ++q) p *= h;
-      ctl->c[threadIdx.x] = threadIdx.x == 0 ? 1.0 : dpp_c(threadIdx.x) * p;
+      for (int q = 0; q < (int)threadIdx.x; ++q) p = scaled ? h : p * h;
+      const double c = threadIdx.x == 0 ? 1.0 : dpp_c(threadIdx.x);
+      ctl->c[threadIdx.x] = c * p;
       ctl->e[threadIdx.x] = dpp_e(threadIdx.x) * (threadIdx.x == 7 ? h : p);
+      ctl->l[threadIdx.x] = scaled ? c : c * p;
     }
   }
 };
@@ -392,7 +404,7 @@ __global__ void __launch_bounds__(kAdjBlock, 1) adjoint_forward_kernel(const __g
         err = sw;
       }
       // v_1; the accepted state becomes rho
-      const double c1 = ctl->c[1], e1 = ctl->e[1];
+      const double c1 = ctl->c[1], e1 = ctl->e[1], hs = ctl->h;
       if (first || accepted) {
         A.each([&](int e, int i, int j) { rho[e] = y1[i * ld + j]; });
       }
@@ -402,29 +414,37 @@ __global__ void __launch_bounds__(kAdjBlock, 1) adjoint_forward_kernel(const __g
         A.each([&](int e, int i, int j) { A.put(y1, i, j, rho[e]); });
         __syncthreads();
       }
-      if (threadIdx.x < d) dq = c1 * A.trace_rows(a.op_p2, y1);
-      A.each([&](int e, int i, int j) {
-        const double2 g = v1[e];
-        sum[e] = vmul(c1, g);
-        err[e] = vmul(e1, g);
-        A.put(y0, i, j, g);
-      });
-      __syncthreads();
-#pragma unroll 1
-      for (int k = 2; k <= 6; ++k) {
-        const double2 *in = (k & 1) ? y1 : y0;
-        double2 *nxt = (k & 1) ? y0 : y1;
-        const double c = ctl->c[k], ce = ctl->e[k];
-        if (threadIdx.x < d) dq = fma(c, A.trace_rows(a.op_p2, in), dq);
+      auto powers = [&](auto scaled) {
+        constexpr bool SC = decltype(scaled)::value;  // dpp_scaled
+        if (threadIdx.x < d) dq = c1 * A.trace_rows(a.op_p2, y1);
         A.each([&](int e, int i, int j) {
-          const double2 g = A.gen(A.drive(Dst[e], w, i, j), w, in, i, j);
-          const double2 sk = vfma(c, g, sum[e]);
-          sum[e] = sk;
-          if (!a.fixed) err[e] = vfma(ce, g, err[e]);
-          A.put(nxt, i, j, k == 6 ? vadd(rho[e], sk) : g);
+          const double2 g = v1[e];
+          sum[e] = vmul(c1, g);
+          err[e] = vmul(e1, g);
+          A.put(y0, i, j, g);
         });
+        if constexpr (SC) A.scale(y0, hs);
         __syncthreads();
-      }
+#pragma unroll 1
+        for (int k = 2; k <= 6; ++k) {
+          const double2 *in = (k & 1) ? y1 : y0;
+          double2 *nxt = (k & 1) ? y0 : y1;
+          const double c = ctl->c[k], ce = ctl->e[k];
+          if (threadIdx.x < d) dq = fma(c, A.trace_rows(a.op_p2, in), dq);
+          A.each([&](int e, int i, int j) {
+            const double2 g = A.gen(A.drive(Dst[e], w, i, j), w, in, i, j);
+            const double2 sk = vfma(c, g, sum[e]);
+            sum[e] = sk;
+            if (!a.fixed) err[e] = vfma(ce, g, err[e]);
+            A.put(nxt, i, j, k == 6 ? vadd(rho[e], sk) : g);
+          });
+          if constexpr (SC)
+            if (k < 6) A.scale(nxt, hs);
+          __syncthreads();
+        }
+      };
+      if (dpp_scaled(hs)) powers(std::true_type());
+      else powers(std::false_type());
       // F of the new state, fused with the error norm
       {
         const double e7 = ctl->e[7];
@@ -532,38 +552,44 @@ __global__ void __launch_bounds__(kAdjBlock, 1) adjoint_backward_kernel(const __
     S[e] = make_double2(0.0, 0.0);
   });
   for (int k = 0; k < nk; ++k) gk[k * kAdjBlock + threadIdx.x] = 0.0;
-  // v_1..v_5 of the step from the state x (already in y1 unless load) into vk;
-  // with xn also the state after a step of length h (its matrix in y1)
-  auto powers_of = [&](double w, const double2 *x, bool load, double2 *vk, double2 *xn) {
+  // v_1..v_5 of the step of length h from the state x (already in y1 unless
+  // load) into vk; with xn also the state after the step (its matrix in y1)
+  auto powers_of = [&](double w, double h, const double2 *x, bool load, double2 *vk, double2 *xn) {
     if (load) {
       __syncthreads();
       A.each([&](int e, int i, int j) { A.put(y1, i, j, x[e]); });
       __syncthreads();
     }
+    auto powers = [&](auto scaled) {
+      constexpr bool SC = decltype(scaled)::value;  // dpp_scaled
 #pragma unroll 1
-    for (int k = 1; k <= (xn ? 6 : 5); ++k) {
-      const double2 *in = (k & 1) ? y1 : y0;
-      double2 *nxt = (k & 1) ? y0 : y1;
-      const double c = ctl->c[k];
-      A.each([&](int e, int i, int j) {
-        const double2 g = A.gen(A.drive(Dst[e], w, i, j), w, in, i, j);
-        if (xn) {
-          const double2 sk = k == 1 ? vmul(c, g) : vfma(c, g, sum[e]);
-          if (k < 6) {
-            sum[e] = sk;
-          } else {
-            const double2 y = vadd(x[e], sk);
-            xn[e] = y;
-            A.put(y1, i, j, y);
+      for (int k = 1; k <= (xn ? 6 : 5); ++k) {
+        const double2 *in = (k & 1) ? y1 : y0;
+        double2 *nxt = (k & 1) ? y0 : y1;
+        const double c = ctl->c[k];
+        A.each([&](int e, int i, int j) {
+          const double2 g = A.gen(A.drive(Dst[e], w, i, j), w, in, i, j);
+          if (xn) {
+            const double2 sk = k == 1 ? vmul(c, g) : vfma(c, g, sum[e]);
+            if (k < 6) {
+              sum[e] = sk;
+            } else {
+              const double2 y = vadd(x[e], sk);
+              xn[e] = y;
+              A.put(y1, i, j, y);
+            }
           }
-        }
-        if (k < 6) {
-          vk[(int64_t)(k - 1) * nent + e] = g;
-          if (k < 5 || xn) A.put(nxt, i, j, g);
-        }
-      });
-      __syncthreads();
-    }
+          if (k < 6) {
+            const double2 v = SC ? vmul(h, g) : g;
+            vk[(int64_t)(k - 1) * nent + e] = v;
+            if (k < 5 || xn) A.put(nxt, i, j, v);
+          }
+        });
+        __syncthreads();
+      }
+    };
+    if (dpp_scaled(h)) powers(std::true_type());
+    else powers(std::false_type());
   };
   double v[2];
   for (int s = a.n_seg - 1; s >= 0; --s) {
@@ -581,7 +607,7 @@ __global__ void __launch_bounds__(kAdjBlock, 1) adjoint_backward_kernel(const __
       if (threadIdx.x < 32) A.powers(hs[m]);
       __syncthreads();
       double2 *x = X + (int64_t)m * nent;
-      powers_of(w, x, false, m < kept ? V + (int64_t)m * 5 * nent : one,
+      powers_of(w, hs[m], x, false, m < kept ? V + (int64_t)m * 5 * nent : one,
                 m + 1 < ns ? x + nent : nullptr);
     }
     double gom = 0.0;
@@ -593,7 +619,7 @@ __global__ void __launch_bounds__(kAdjBlock, 1) adjoint_backward_kernel(const __
       if (threadIdx.x < 32) A.powers(h);
       __syncthreads();
       if (m >= kept) {
-        if (m + 1 < ns) powers_of(w, x, true, one, nullptr);
+        if (m + 1 < ns) powers_of(w, h, x, true, one, nullptr);
         vk = one;
       }
       {
@@ -602,56 +628,63 @@ __global__ void __launch_bounds__(kAdjBlock, 1) adjoint_backward_kernel(const __
         A.each([&](int e, int i, int j) { A.put(y0, i, j, vmul(c6, lam[e])); });
         __syncthreads();
       }
-      // a_k in y0 (k even) or y1 (k odd)
+      // a_k (of a scaled step: a_k / h^(k-1)) in y0 (k even) or y1 (k odd)
+      auto adjoint = [&](auto scaled) {
+        constexpr bool SC = decltype(scaled)::value;  // dpp_scaled
 #pragma unroll 1
-      for (int k = 6; k >= 1; --k) {
-        const double2 *in = (k & 1) ? y1 : y0;
-        double2 *nxt = (k & 1) ? y0 : y1;
-        const double2 *vp = k == 1 ? x : vk + (int64_t)(k - 2) * nent;
-        const double cl = ctl->c[k - 1], cp = ctl->c[k];
-        A.each([&](int e, int i, int j) {
-          const double wt = A.weight(i, j);
-          const double2 av = in[i * ld + j], y = vp[e];
-          double2 yw = make_double2(wt * y.x, wt * y.y);
-          // the diagonal of F^dag, and conj(a) v for its parameter derivatives
-          double2 o = make_double2(0.0, 0.0), sv = S[e];
-          cmac(o, cj(A.drive(Dst[e], w, i, j)), av);
-          sv.x = fma(av.x, yw.x, sv.x);
-          sv.x = fma(av.y, yw.y, sv.x);
-          if (a.dk_complex) {
-            sv.y = fma(av.x, yw.y, sv.y);
-            sv.y = fma(-av.y, yw.x, sv.y);
-          }
-          S[e] = sv;
-          double2 z = make_double2(0.0, 0.0);
-          if (a.op_hd.w > 0) {
-            z = A.commutator(a.op_hd, in, i, j);
-            o.x = fma(-w, z.y, o.x);  // +i w z
-            o.y = fma(w, z.x, o.y);
-          }
-          if (a.hd_diag) z = vfma(a.diag_h[i].y - a.diag_h[j].y, av, z);
-          gom = fma(-z.y, yw.x, gom);  // <i z, v>
-          gom = fma(z.x, yw.y, gom);
-          if (a.op_h0.w > 0) {
-            const double2 c = A.commutator(a.op_h0, in, i, j);
-            o.x -= c.y;
-            o.y += c.x;
-          }
-          for (int q = 0; q < nk; ++q)
-            if (a.op_a[q].w > 0 || a.op_n[q].w > 0) {
-              const double2 t = A.dissipator(q, true, in, i, j);
-              o = vfma(A.gam[q], t, o);
-              double g = gk[q * kAdjBlock + threadIdx.x];
-              g = fma(t.x, yw.x, g);
-              gk[q * kAdjBlock + threadIdx.x] = fma(t.y, yw.y, g);
+        for (int k = 6; k >= 1; --k) {
+          const double2 *in = (k & 1) ? y1 : y0;
+          double2 *nxt = (k & 1) ? y0 : y1;
+          const double2 *vp = k == 1 ? x : vk + (int64_t)(k - 2) * nent;
+          const double cl = ctl->l[k - 1], cp = ctl->c[k];
+          A.each([&](int e, int i, int j) {
+            const double wt = A.weight(i, j);
+            const double2 av = in[i * ld + j], y = vp[e];
+            double2 yw = make_double2(wt * y.x, wt * y.y);
+            // the diagonal of F^dag, and conj(a) v for its parameter derivatives
+            double2 o = make_double2(0.0, 0.0), sv = S[e];
+            cmac(o, cj(A.drive(Dst[e], w, i, j)), av);
+            sv.x = fma(av.x, yw.x, sv.x);
+            sv.x = fma(av.y, yw.y, sv.x);
+            if (a.dk_complex) {
+              sv.y = fma(av.x, yw.y, sv.y);
+              sv.y = fma(-av.y, yw.x, sv.y);
             }
-          o = vfma(cl, lam[e], o);
-          o = vfma(cp, P2[e], o);
-          if (k == 1) lam[e] = o;
-          else A.put(nxt, i, j, o);
-        });
-        __syncthreads();
-      }
+            S[e] = sv;
+            double2 z = make_double2(0.0, 0.0);
+            if (a.op_hd.w > 0) {
+              z = A.commutator(a.op_hd, in, i, j);
+              o.x = fma(-w, z.y, o.x);  // +i w z
+              o.y = fma(w, z.x, o.y);
+            }
+            if (a.hd_diag) z = vfma(a.diag_h[i].y - a.diag_h[j].y, av, z);
+            gom = fma(-z.y, yw.x, gom);  // <i z, v>
+            gom = fma(z.x, yw.y, gom);
+            if (a.op_h0.w > 0) {
+              const double2 c = A.commutator(a.op_h0, in, i, j);
+              o.x -= c.y;
+              o.y += c.x;
+            }
+            for (int q = 0; q < nk; ++q)
+              if (a.op_a[q].w > 0 || a.op_n[q].w > 0) {
+                const double2 t = A.dissipator(q, true, in, i, j);
+                o = vfma(A.gam[q], t, o);
+                double g = gk[q * kAdjBlock + threadIdx.x];
+                g = fma(t.x, yw.x, g);
+                gk[q * kAdjBlock + threadIdx.x] = fma(t.y, yw.y, g);
+              }
+            o = vfma(cl, lam[e], o);
+            o = vfma(cp, P2[e], o);
+            if (k == 1) lam[e] = o;
+            else A.put(nxt, i, j, o);
+          });
+          if constexpr (SC)
+            if (k > 1) A.scale(nxt, h);
+          __syncthreads();
+        }
+      };
+      if (dpp_scaled(h)) adjoint(std::true_type());
+      else adjoint(std::false_type());
     }
     v[0] = gom;
     A.reduce(v, 1);

@@ -203,6 +203,12 @@ template <> struct DPW<float> {
 // (the low orders of the error cancel against L ynew).  Six products per step
 // as before, but no stage combinations: 13 multiply-adds per component and
 // step instead of 33.
+// With h |L| of order one, h^6 and L^6 y both stay in the FP64 range while h
+// lies within 2^-128 .. 2^128.  A step of another length (dpp_scaled) takes
+// v_k = h L v_(k-1): the factor h is applied to a vector after the products with
+// L of the whole system are formed, in a pass or code of its own.  (Under a
+// condition within the common code it cost 5 to 12 % of the FP64 kernels' time:
+// the FP64 pipe carries a multiplication out whether or not its predicate holds.)
 struct DPP {
   static constexpr double c2 = 1.0 / 2, c3 = 1.0 / 6, c4 = 1.0 / 24, c5 = 1.0 / 120,
                           c6 = 1.0 / 600;  // c_1 = 1
@@ -215,6 +221,11 @@ __host__ __device__ constexpr double dpp_c(int k) {
 __host__ __device__ constexpr double dpp_e(int k) {
   return k == 1 ? DPP::e1 : k == 2 ? DPP::e2 : k == 3 ? DPP::e3 : k == 4 ? DPP::e4
        : k == 5 ? DPP::e5 : k == 6 ? DPP::e6 : DPP::e7;
+}
+
+__device__ __forceinline__ bool dpp_scaled(double h) {
+  const int hi = __double2hiint(h);
+  return hi < ((1023 - 128) << 20) || hi >= ((1023 + 128) << 20);
 }
 
 // a < b for values that are not negative, by their integer order (an FP64

@@ -824,31 +824,39 @@ struct Traj {
       // divisions, pow and sqrt were two thirds of its 480 per step
       // (Jaynes-Cummings, dim 20).  500 trajectories 191 -> 89 ms.
       // k[1], k[2]: the sums of the step and of the error; k[3]: v_(j+1).
-      double hp = ht;
-#pragma unroll
-      for (int q = 0; q < R; ++q) {
-        yt[q] = k[0][q];
-        k[1][q] = vmul(hp, yt[q]);
-        k[2][q] = vmul(DPP::e1 * hp, yt[q]);
-      }
-      auto power = [&](auto copy, int j, bool lead) {
-        rhs_f<false, decltype(copy)::value>(yt, k[3], u0, (T)0, 0, lead);
-        hp *= ht;
-        const double c = dpp_c(j) * hp, e = dpp_e(j) * hp;
+      auto powers = [&](auto scaled) {
+        constexpr bool SC = decltype(scaled)::value;  // dpp_scaled
+        const double hm = SC ? 1.0 : (double)ht;
+        double hp = hm;
 #pragma unroll
         for (int q = 0; q < R; ++q) {
-          yt[q] = k[3][q];
-          k[1][q] = vfma(c, yt[q], k[1][q]);
-          if (want_err) k[2][q] = vfma(e, yt[q], k[2][q]);
+          yt[q] = k[0][q];
+          if constexpr (SC) yt[q] = vmul(ht, yt[q]);
+          k[1][q] = vmul(hp, yt[q]);
+          k[2][q] = vmul(DPP::e1 * hp, yt[q]);
         }
+        auto power = [&](auto copy, int j, bool lead) {
+          rhs_f<false, decltype(copy)::value>(yt, k[3], u0, (T)0, 0, lead);
+          hp *= hm;
+          const double c = dpp_c(j) * hp, e = dpp_e(j) * hp;
+#pragma unroll
+          for (int q = 0; q < R; ++q) {
+            yt[q] = k[3][q];
+            if constexpr (SC) yt[q] = vmul(ht, yt[q]);
+            k[1][q] = vfma(c, yt[q], k[1][q]);
+            if (want_err) k[2][q] = vfma(e, yt[q], k[2][q]);
+          }
+        };
+        const std::integral_constant<int, 0> c0;
+        const std::integral_constant<int, 1> c1;
+        power(c0, 2, !want_err);
+        power(c1, 3, false);
+        power(c0, 4, false);
+        power(c1, 5, false);
+        power(c0, 6, false);
       };
-      const std::integral_constant<int, 0> c0;
-      const std::integral_constant<int, 1> c1;
-      power(c0, 2, !want_err);
-      power(c1, 3, false);
-      power(c0, 4, false);
-      power(c1, 5, false);
-      power(c0, 6, false);
+      if (dpp_scaled(ht)) powers(std::true_type());
+      else powers(std::false_type());
 #pragma unroll
       for (int q = 0; q < R; ++q) {
         ynew[q] = vadd(psi[q], k[1][q]);

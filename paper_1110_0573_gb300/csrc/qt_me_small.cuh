@@ -35,6 +35,7 @@
 #pragma once
 
 #include <cooperative_groups.h>
+#include <type_traits>
 
 #include "qt_device.cuh"
 #include "qt_internal.h"
@@ -96,8 +97,9 @@ constexpr size_t kSmallSmemMax = kSmemPerCta - 1024;
 // What warp 0 of each CTA hands to the others after each step attempt.
 struct SmallCtl {
   double h;      // length of the next attempt
-  double c[8];   // FP64: c_k h^k
-  double e[8];   // FP64: e_k h^k
+  // FP64: the weights of L v_(k-1), c_k h^k and e_k h^k (dpp_scaled: c_k h and
+  // e_k h); e_7 h
+  double c[8], e[8];
   int accepted;  // the last attempt was accepted (its state is in y1)
   int out;       // output index to write from y1, or -1
   int done;
@@ -525,7 +527,8 @@ struct SmallSolver {
       if (!done && !skip) next();
       if (sizeof(T) == 8 && threadIdx.x >= 1 && threadIdx.x <= 7) {  // coefficients of v_k
         double p = h;
-        for (int q = 1; q < (int)threadIdx.x; ++q) p *= h;
+        if (!dpp_scaled(h))
+          for (int q = 1; q < (int)threadIdx.x; ++q) p *= h;
         ctl->c[threadIdx.x] = dpp_c(threadIdx.x) * p;
         // L ynew takes one power of h
         ctl->e[threadIdx.x] = dpp_e(threadIdx.x) * (threadIdx.x == 7 ? h : p);
@@ -566,36 +569,48 @@ struct SmallSolver {
       // FP32 power of a large generator would overflow) with c_k, e_k
       auto ck = [&](int q) { return sizeof(T) == 8 ? (T)ctl->c[q] : (T)dpp_c(q); };
       auto ek = [&](int q) { return sizeof(T) == 8 ? (T)ctl->e[q] : (T)dpp_e(q); };
-      // v_1; the accepted state becomes rho
-      {
-        const T c = ck(1), ce = ek(1);
-        each([&](int l, int i, int j) {
-          const V r = accepted ? y1[i * ld + j] : rho[l];
-          if (accepted) rho[l] = r;
-          V g = v1[l];
-          if constexpr (sizeof(T) == 4) g = vmul(ht, g);
-          sum[l] = vmul(c, g);
-          err[l] = vmul(ce, g);
-          put(y0, i, j, g);
-        });
-      }
-      sync();
-      // v_2 .. v_6, the last fused with the new state (into y1)
-#pragma unroll 1
-      for (int q = 2; q <= 6; ++q) {
-        const V *in = (q & 1) ? y1 : y0;
-        V *nxt = (q & 1) ? y0 : y1;
-        const T c = ck(q), ce = ek(q);
-        each([&](int l, int i, int j) {
-          V g = f(in, l, i, j);
-          if constexpr (sizeof(T) == 4) g = vmul(ht, g);
-          const V s = vfma(c, g, sum[l]);
-          sum[l] = s;
-          err[l] = vfma(ce, g, err[l]);
-          put(nxt, i, j, q == 6 ? vadd(rho[l], s) : g);
-        });
+      auto powers = [&](auto scaled) {
+        constexpr bool SC = decltype(scaled)::value;  // FP64: dpp_scaled
+        // this thread's entries of a vector by h
+        auto scale = [&](V *buf) {
+          each([&](int, int i, int j) { put(buf, i, j, vmul(ht, buf[i * ld + j])); });
+        };
+        // v_1; the accepted state becomes rho
+        {
+          const T c = ck(1), ce = ek(1);
+          each([&](int l, int i, int j) {
+            const V r = accepted ? y1[i * ld + j] : rho[l];
+            if (accepted) rho[l] = r;
+            V g = v1[l];
+            if constexpr (sizeof(T) == 4) g = vmul(ht, g);
+            sum[l] = vmul(c, g);
+            err[l] = vmul(ce, g);
+            put(y0, i, j, g);
+          });
+          if constexpr (SC) scale(y0);
+        }
         sync();
-      }
+        // v_2 .. v_6, the last fused with the new state (into y1)
+#pragma unroll 1
+        for (int q = 2; q <= 6; ++q) {
+          const V *in = (q & 1) ? y1 : y0;
+          V *nxt = (q & 1) ? y0 : y1;
+          const T c = ck(q), ce = ek(q);
+          each([&](int l, int i, int j) {
+            V g = f(in, l, i, j);
+            if constexpr (sizeof(T) == 4) g = vmul(ht, g);
+            const V s = vfma(c, g, sum[l]);
+            sum[l] = s;
+            err[l] = vfma(ce, g, err[l]);
+            put(nxt, i, j, q == 6 ? vadd(rho[l], s) : g);
+          });
+          if constexpr (SC)
+            if (q < 6) scale(nxt);
+          sync();
+        }
+      };
+      if (sizeof(T) == 8 && dpp_scaled((double)ht)) powers(std::true_type());
+      else powers(std::false_type());
       // L ynew fused with the error norm
       {
         const T at = (T)a.atol, rt = (T)a.rtol;
