@@ -23,8 +23,10 @@ namespace {
 
 constexpr int kBatchWarps = kBatchBlock / 32;
 
-// Dynamic shared memory per CTA: two CTAs per SM for the mixed kernel, one
-// for the FP64 kernel.
+// Dynamic shared memory per CTA at most: two CTAs per SM for the mixed kernel,
+// one for the FP64 kernel.  A launch takes what its largest problem needs
+// (batch_smem_*): the rest of the SM's memory is its L1 cache, through which the
+// Monte-Carlo items read their collapse and observable operators.
 template <typename T> constexpr size_t kBatchSmem = sizeof(T) == 4 ? 112 * 1024 : 224 * 1024;
 
 // The CTA's current item, then one of: the Monte-Carlo items' buffers, the
@@ -152,7 +154,7 @@ __global__ void __launch_bounds__(kBatchBlock, (sizeof(T) == 4 ? 2 : 1)) batch_k
       const bool herm = P.state_is_ket != 0;
       const int d = P.ops.d, nent = small_entries(d, herm);
       unsigned char *region = dyn + kBatchItemBytes;
-      constexpr size_t room = kBatchSmem<T> - kBatchItemBytes;
+      const size_t room = a.smem - kBatchItemBytes;
       const size_t base = small_smem(prec, d, nent, P.small, 1, kBatchBlock, false).total;
       if (2 * P.small.nl + P.small.kc <= kSmallTerms && base <= room) {
         // the entry arrays after the solver's shared memory when they fit
@@ -269,11 +271,26 @@ size_t batch_ws_stride(int dmax, int precision) {
   return ((11 * (size_t)dmax * dmax * elem + 255) / 256) * 256;
 }
 
+size_t batch_smem_mc(int precision) {
+  return kBatchItemBytes + (precision == QT_MIXED ? sizeof(BatchShared<float>) : sizeof(BatchShared<double>));
+}
+
+size_t batch_smem_me(int precision, int d, SmallInfo f, bool is_ket, bool arrays) {
+  const size_t room =
+      (precision == QT_MIXED ? kBatchSmem<float> : kBatchSmem<double>) - kBatchItemBytes;
+  const int nent = small_entries(d, is_ket);
+  const size_t base = small_smem(precision, d, nent, f, 1, kBatchBlock, false).total;
+  if (2 * f.nl + f.kc > kSmallTerms || base > room)  // the general solver
+    return kBatchItemBytes + sizeof(BatchMeShared);
+  const size_t all = base + small_ws_bytes(precision, d, nent, f, 1, kBatchBlock);
+  return kBatchItemBytes + (arrays && all <= room ? all : base);
+}
+
 cudaError_t launch_batch(const BatchArgs &a, int precision, int grid, cudaStream_t s) {
   if (precision == QT_MIXED)
-    batch_kernel<float><<<grid, kBatchBlock, kBatchSmem<float>, s>>>(a);
+    batch_kernel<float><<<grid, kBatchBlock, a.smem, s>>>(a);
   else
-    batch_kernel<double><<<grid, kBatchBlock, kBatchSmem<double>, s>>>(a);
+    batch_kernel<double><<<grid, kBatchBlock, a.smem, s>>>(a);
   return cudaGetLastError();
 }
 

@@ -1544,6 +1544,7 @@ struct qt_batch_s {
   unsigned long long *prob_ctl = nullptr;   // [n][6] statistics per problem
   void *ws = nullptr;
   size_t ws_stride = 0;
+  size_t smem[2] = {0, 0};                  // shared memory per CTA: QT_FP64, QT_MIXED
   int grid = 0;
   ~qt_batch_s() {
     for (void *p : dev)
@@ -1771,6 +1772,23 @@ int qt_batch_create(const qt_problem *problems, int n_problems, qt_batch *out) {
   const int g64 = qt::batch_grid(QT_FP64), g32 = qt::batch_grid(QT_MIXED);
   b->grid = std::max(g64, g32);
   b->ws_stride = qt::batch_ws_stride(b->dmax, QT_FP64);
+  // the shared memory of a launch: that of its largest problem; in mixed
+  // precision without the entry arrays of the master-equation items (they go to
+  // the workspace then) when a Monte-Carlo problem has wide operators
+  bool wide = false;
+  for (int p = 0; p < n_problems; ++p) {
+    if (problems[p].kind != QT_KIND_MC) continue;
+    const int64_t end = p + 1 < n_problems ? off_all[info[p + 1].wbase] : (int64_t)cols.size();
+    const int64_t h = off_all[info[p].wbase] + (int64_t)w_all[info[p].wbase] * info[p].d;
+    wide = wide || (end - h) * (int64_t)(sizeof(float2) + sizeof(int)) > qt::kBatchWideOps;
+  }
+  for (int prec : {QT_FP64, QT_MIXED})
+    for (int p = 0; p < n_problems; ++p)
+      b->smem[prec] = std::max(
+          b->smem[prec], problems[p].kind == QT_KIND_MC
+                             ? qt::batch_smem_mc(prec)
+                             : qt::batch_smem_me(prec, info[p].d, infos[p], probs[p].state_is_ket != 0,
+                                                 prec == QT_FP64 || !wide));
   for (int p = 0; p < n_problems; ++p) {  // and the small solver's workspace
     if (problems[p].kind != QT_KIND_ME) continue;
     qt::MeArgs m;
@@ -1847,6 +1865,7 @@ int qt_batch_solve_dev(qt_batch b, const double *tlist_dev, int n_t, const qt_op
   a.ws = b->ws;
   a.ws_stride = b->ws_stride;
   a.small_group_dim = b->small_group_dim;
+  a.smem = b->smem[o->precision];
   const int grid = qt::batch_grid(o->precision);
   if (grid <= 0) return fail(QT_ECUDA, "cannot size the batch launch");
   QT_CK(qt::launch_batch(a, o->precision, std::min(grid, b->grid), st));

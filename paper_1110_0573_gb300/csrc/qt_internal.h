@@ -274,12 +274,27 @@ struct BatchArgs {
   void *ws;                       // master-equation workspace, ws_stride bytes per CTA
   size_t ws_stride;
   int small_group_dim;            // MC items up to this dimension: half-warp groups
+  size_t smem;                    // dynamic shared memory per CTA (batch_smem)
 };
 
 constexpr int kBatchBlock = 256;
 
 cudaError_t launch_batch(const BatchArgs &a, int precision, int grid, cudaStream_t s);
 int batch_grid(int precision);
+// Shared memory per CTA that a problem needs: a Monte-Carlo problem, or a
+// master-equation problem of the given structure (with its entry arrays when
+// they fit and arrays is set).
+size_t batch_smem_mc(int precision);
+size_t batch_smem_me(int precision, int d, SmallInfo f, bool is_ket, bool arrays);
+// Bytes of collapse and observable operators from which a Monte-Carlo item of
+// the mixed kernel wants the L1 cache that two CTAs with the master-equation
+// items' arrays leave (28 KB).  256 problems of 256 trajectories on 41 against
+// 112 KB per CTA: 6.9 KB of operators 7.12 / 7.11 ms, 13 KB 8.16 / 10.1 (dim 32)
+// and 11.5 / 15.5 (dim 64).  256 master equations of dim 32 beside four such
+// problems, their arrays in the workspace / in shared memory: 2.23 / 2.68 ms (5.3
+// / 6.9 at dim 64); 512 beside one of 16 trajectories: 2.40 / 2.28.  (FP64: one
+// CTA per SM, at most 2 %.)
+constexpr int64_t kBatchWideOps = 8 * 1024;
 size_t batch_ws_stride(int dmax, int precision);
 cudaError_t launch_batch_finalize(const BatchArgs &a, cudaStream_t s);
 
