@@ -243,8 +243,10 @@ int qt_mcsolve_td(const qt_op *H, const qt_td *td, const qt_op *c_ops, int n_c,
  * (QT_EINVAL otherwise).  corr_out[n_t * n_tau] (host): C(t_k, tau_j) at
  * [k * n_tau + j].  td nullable (time-dependent terms as in qt_mesolve_td;
  * the tau evolution of X_k then sees H(t_k + tau)).  The first solve uses
- * o->me_method; the tau evolutions run the general solver (QT_ME_DENSE_TC is
- * taken as QT_ME_AUTO there).  stats (nullable) sums both stages.
+ * o->me_method; the tau evolutions assume no symmetry of X_k (QT_ME_DENSE_TC
+ * is taken as QT_ME_AUTO there): dim <= 64 by the small-system solver
+ * (time-independent, at most 64 terms per entry), else by the general one.
+ * stats (nullable) sums both stages.
  */
 int qt_correlation_2op_2t(const qt_op *H, const qt_td *td, const qt_op *c_ops, int n_c,
                           const qt_op *A, const qt_op *B, const qt_c128 *state0, int state_is_ket,
@@ -301,8 +303,9 @@ int qt_propagator_steadystate(const qt_op *H, const qt_op *c_ops, int n_c, const
  * maps row-major vec(rho(tlist[0])) to vec(rho(tlist[k])) for Eq.
  * (master_equation) with H (plus the time-dependent terms td, nullable) and
  * c_ops; U(t_0) = I.  Column a dim + b is the solution from the matrix unit
- * E_ab, computed on the GPU one CTA per unit with the general solver and the
- * options o (precision, tolerances; QT_ME_DENSE_TC is taken as QT_ME_AUTO).
+ * E_ab, computed on the GPU one CTA per unit as a tau evolution of
+ * qt_correlation_2op_2t, with the options o (precision, tolerances;
+ * QT_ME_DENSE_TC is taken as QT_ME_AUTO).
  * Built for dim <= 64 (QT_ENOTIMPL above); stats sums the dim^2 solves.
  */
 int qt_propagator(const qt_op *H, const qt_td *td, const qt_op *c_ops, int n_c,

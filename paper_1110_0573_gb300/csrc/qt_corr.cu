@@ -78,8 +78,8 @@ __device__ void cta_solve(const MeArgs &m) {
 
 // CTA b evolves X_k for k = b, b + grid, ...; its slab of a.work holds the
 // solver workspace, X_k and the times.  a carries the tau evolution (n_t =
-// n_tau, expect = the correlation array, general solver).
-// MODE: the solver of the CTA (SmallMode below).
+// n_tau, expect = the correlation array, all d*d entries of X_k).
+// MODE: the solver of the CTA (SmallMode above).
 template <typename T, SmallMode MODE>
 __global__ void __launch_bounds__(kMeBlock) corr_block_kernel(const __grid_constant__ MeArgs a,
                                                               const __grid_constant__ CorrArgs c) {
@@ -103,7 +103,7 @@ __global__ void __launch_bounds__(kMeBlock) corr_block_kernel(const __grid_const
 }
 
 // The propagator: CTA b evolves the matrix units E_k (k = a d + b') for
-// k = b, b + grid, ... from tlist[0] by the general solver and scatters each
+// k = b, b + grid, ... from tlist[0] by the solver of MODE and scatters each
 // output state rho_k(t_m) into column k of U(t_m): U[m][ij][k].
 template <typename T, SmallMode MODE>
 __global__ void __launch_bounds__(kMeBlock) prop_block_kernel(const __grid_constant__ MeArgs a,

@@ -159,7 +159,7 @@ constexpr int kCSlotsMax = 32;
 constexpr int kCTermsMax = 512;
 
 constexpr int kMeBlock = 256;
-constexpr int kMeSmallDim = 64;  // systems up to this dimension are solved by one CTA
+constexpr int kMeSmallDim = 64;  // systems up to this dimension are solved by one CTA or cluster
 
 // Steady state (qt_ss.cu): GMRES(m) on A(x) = L(x) + w Tr(x) I.
 constexpr int kGmBlock = 512;
