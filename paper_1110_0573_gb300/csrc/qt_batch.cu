@@ -156,7 +156,7 @@ __global__ void __launch_bounds__(kBatchBlock, (sizeof(T) == 4 ? 2 : 1)) batch_k
       unsigned char *region = dyn + kBatchItemBytes;
       const size_t room = a.smem - kBatchItemBytes;
       const size_t base = small_smem(prec, d, nent, P.small, 1, kBatchBlock, false).total;
-      if (2 * P.small.nl + P.small.kc <= kSmallTerms && base <= room) {
+      if (small_takes(P.small) && base <= room) {
         // the entry arrays after the solver's shared memory when they fit
         unsigned char *work =
             base + small_ws_bytes(prec, d, nent, P.small, 1, kBatchBlock) <= room
@@ -280,7 +280,7 @@ size_t batch_smem_me(int precision, int d, SmallInfo f, bool is_ket, bool arrays
       (precision == QT_MIXED ? kBatchSmem<float> : kBatchSmem<double>) - kBatchItemBytes;
   const int nent = small_entries(d, is_ket);
   const size_t base = small_smem(precision, d, nent, f, 1, kBatchBlock, false).total;
-  if (2 * f.nl + f.kc > kSmallTerms || base > room)  // the general solver
+  if (!small_takes(f) || base > room)  // the general solver
     return kBatchItemBytes + sizeof(BatchMeShared);
   const size_t all = base + small_ws_bytes(precision, d, nent, f, 1, kBatchBlock);
   return kBatchItemBytes + (arrays && all <= room ? all : base);

@@ -204,11 +204,12 @@ template <> struct DPW<float> {
 // as before, but no stage combinations: 13 multiply-adds per component and
 // step instead of 33.
 // With h |L| of order one, h^6 and L^6 y both stay in the FP64 range while h
-// lies within 2^-128 .. 2^128.  A step of another length (dpp_scaled) takes
-// v_k = h L v_(k-1): the factor h is applied to a vector after the products with
-// L of the whole system are formed, in a pass or code of its own.  (Under a
-// condition within the common code it cost 5 to 12 % of the FP64 kernels' time:
-// the FP64 pipe carries a multiplication out whether or not its predicate holds.)
+// lies within 2^-128 .. 2^128.  A trajectory or adjoint step of another length
+// (dpp_scaled) takes v_k = h L v_(k-1), in code of its own: the FP64 pipe
+// carries a multiplication out whether or not its predicate holds, and under a
+// condition within the common code those cost 5 to 12 % of the kernels' time.
+// (The small-system solver leaves such generators to the general one, which
+// keeps the stages: SmallInfo::in_range.)
 struct DPP {
   static constexpr double c2 = 1.0 / 2, c3 = 1.0 / 6, c4 = 1.0 / 24, c5 = 1.0 / 120,
                           c6 = 1.0 / 600;  // c_1 = 1

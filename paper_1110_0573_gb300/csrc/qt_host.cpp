@@ -374,10 +374,20 @@ int ell_append(const Csr &A, std::vector<int> &cols, std::vector<double2> &vals,
   return w;
 }
 
+// The powers of the generator that FP64 steps take (DPP in qt_device.cuh) stay
+// in range: its largest entry is within 2^-100 .. 2^100.
+bool generator_in_range(const Csr &heff, const std::vector<Csr> &C) {
+  double m = 0.0;
+  for (const cplx &v : heff.val) m = std::max({m, std::abs(v.real()), std::abs(v.imag())});
+  for (const Csr &c : C)  // (their squares are the terms of the generator)
+    for (const cplx &v : c.val) m = std::max(m, std::norm(v));
+  return m >= 0x1p-100 && m <= 0x1p100;
+}
+
 // Structure of H_eff and the collapse operators for the small-system solver;
 // a collapse operator's ELL width is its longest row, at least 1.
 qt::SmallInfo small_info(const Csr &heff, const std::vector<Csr> &C) {
-  qt::SmallInfo f = {0, 0, 1, 1};
+  qt::SmallInfo f = {0, 0, 1, 1, generator_in_range(heff, C) ? 1 : 0};
   for (int i = 0; i < heff.d; ++i) {
     int n = 0;
     for (int64_t p = heff.ptr[i]; p < heff.ptr[i + 1]; ++p)

@@ -108,6 +108,7 @@ struct SmallInfo {
   int kc;     // sum of squared ELL widths of the collapse operators that are not diagonal
   int hreal;  // every off-diagonal entry of H_eff is real
   int creal;  // every entry of those collapse operators is real
+  int in_range;  // powers of the generator stay in the FP64 range (DPP, qt_device.cuh)
 };
 
 // Kernel arguments of the master-equation solver.

@@ -35,7 +35,6 @@
 #pragma once
 
 #include <cooperative_groups.h>
-#include <type_traits>
 
 #include "qt_device.cuh"
 #include "qt_internal.h"
@@ -97,9 +96,8 @@ constexpr size_t kSmallSmemMax = kSmemPerCta - 1024;
 // What warp 0 of each CTA hands to the others after each step attempt.
 struct SmallCtl {
   double h;      // length of the next attempt
-  // FP64: the weights of L v_(k-1), c_k h^k and e_k h^k (dpp_scaled: c_k h and
-  // e_k h); e_7 h
-  double c[8], e[8];
+  double c[8];   // FP64: c_k h^k
+  double e[8];   // FP64: e_k h^k
   int accepted;  // the last attempt was accepted (its state is in y1)
   int out;       // output index to write from y1, or -1
   int done;
@@ -159,12 +157,16 @@ __host__ __device__ inline size_t small_ws_bytes(int precision, int d, int nent,
          small_smem(precision, d, nent, f, ranks, threads, true).k;
 }
 
-// Systems that the solver takes: time-independent, with at most kSmallTerms
+// Systems that the solver takes: time-independent, in units in which the powers
+// of the generator are in the FP64 range, with at most kSmallTerms
 // terms per entry (operators with wider rows go to the general solver, which
 // forms their products row by row).
 constexpr int kSmallTerms = 64;
+__host__ __device__ inline bool small_takes(SmallInfo f) {
+  return f.in_range && 2 * f.nl + f.kc <= kSmallTerms;
+}
 inline bool small_fits(const MeArgs &a) {
-  return a.n_td == 0 && a.ops.d <= kMeSmallDim && 2 * a.small.nl + a.small.kc <= kSmallTerms;
+  return a.n_td == 0 && a.ops.d <= kMeSmallDim && small_takes(a.small);
 }
 
 // CTAs of a solve on its own.  A cluster divides the FP64 work but adds about
@@ -527,8 +529,7 @@ struct SmallSolver {
       if (!done && !skip) next();
       if (sizeof(T) == 8 && threadIdx.x >= 1 && threadIdx.x <= 7) {  // coefficients of v_k
         double p = h;
-        if (!dpp_scaled(h))
-          for (int q = 1; q < (int)threadIdx.x; ++q) p *= h;
+        for (int q = 1; q < (int)threadIdx.x; ++q) p *= h;
         ctl->c[threadIdx.x] = dpp_c(threadIdx.x) * p;
         // L ynew takes one power of h
         ctl->e[threadIdx.x] = dpp_e(threadIdx.x) * (threadIdx.x == 7 ? h : p);
@@ -569,48 +570,36 @@ struct SmallSolver {
       // FP32 power of a large generator would overflow) with c_k, e_k
       auto ck = [&](int q) { return sizeof(T) == 8 ? (T)ctl->c[q] : (T)dpp_c(q); };
       auto ek = [&](int q) { return sizeof(T) == 8 ? (T)ctl->e[q] : (T)dpp_e(q); };
-      auto powers = [&](auto scaled) {
-        constexpr bool SC = decltype(scaled)::value;  // FP64: dpp_scaled
-        // this thread's entries of a vector by h
-        auto scale = [&](V *buf) {
-          each([&](int, int i, int j) { put(buf, i, j, vmul(ht, buf[i * ld + j])); });
-        };
-        // v_1; the accepted state becomes rho
-        {
-          const T c = ck(1), ce = ek(1);
-          each([&](int l, int i, int j) {
-            const V r = accepted ? y1[i * ld + j] : rho[l];
-            if (accepted) rho[l] = r;
-            V g = v1[l];
-            if constexpr (sizeof(T) == 4) g = vmul(ht, g);
-            sum[l] = vmul(c, g);
-            err[l] = vmul(ce, g);
-            put(y0, i, j, g);
-          });
-          if constexpr (SC) scale(y0);
-        }
-        sync();
-        // v_2 .. v_6, the last fused with the new state (into y1)
+      // v_1; the accepted state becomes rho
+      {
+        const T c = ck(1), ce = ek(1);
+        each([&](int l, int i, int j) {
+          const V r = accepted ? y1[i * ld + j] : rho[l];
+          if (accepted) rho[l] = r;
+          V g = v1[l];
+          if constexpr (sizeof(T) == 4) g = vmul(ht, g);
+          sum[l] = vmul(c, g);
+          err[l] = vmul(ce, g);
+          put(y0, i, j, g);
+        });
+      }
+      sync();
+      // v_2 .. v_6, the last fused with the new state (into y1)
 #pragma unroll 1
-        for (int q = 2; q <= 6; ++q) {
-          const V *in = (q & 1) ? y1 : y0;
-          V *nxt = (q & 1) ? y0 : y1;
-          const T c = ck(q), ce = ek(q);
-          each([&](int l, int i, int j) {
-            V g = f(in, l, i, j);
-            if constexpr (sizeof(T) == 4) g = vmul(ht, g);
-            const V s = vfma(c, g, sum[l]);
-            sum[l] = s;
-            err[l] = vfma(ce, g, err[l]);
-            put(nxt, i, j, q == 6 ? vadd(rho[l], s) : g);
-          });
-          if constexpr (SC)
-            if (q < 6) scale(nxt);
-          sync();
-        }
-      };
-      if (sizeof(T) == 8 && dpp_scaled((double)ht)) powers(std::true_type());
-      else powers(std::false_type());
+      for (int q = 2; q <= 6; ++q) {
+        const V *in = (q & 1) ? y1 : y0;
+        V *nxt = (q & 1) ? y0 : y1;
+        const T c = ck(q), ce = ek(q);
+        each([&](int l, int i, int j) {
+          V g = f(in, l, i, j);
+          if constexpr (sizeof(T) == 4) g = vmul(ht, g);
+          const V s = vfma(c, g, sum[l]);
+          sum[l] = s;
+          err[l] = vfma(ce, g, err[l]);
+          put(nxt, i, j, q == 6 ? vadd(rho[l], s) : g);
+        });
+        sync();
+      }
       // L ynew fused with the error norm
       {
         const T at = (T)a.atol, rt = (T)a.rtol;
